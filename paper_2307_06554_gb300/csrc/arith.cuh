@@ -24,6 +24,11 @@ __device__ __forceinline__ W csub(W x, W m) {
   return y < x ? y : x;
 }
 
+// 32-bit words: one fused add-and-minimum, min(x - m, x), where the generic
+// form is an addition and a minimum (a Harvey butterfly 7 -> 6 instructions;
+// n = 4096, eight 30-bit primes, 256 products: 65.4 -> 63.6 us)
+__device__ __forceinline__ uint32_t csub(uint32_t x, uint32_t m) { return __viaddmin_u32(x, 0u - m, x); }
+
 __device__ __forceinline__ uint32_t mulhi(uint32_t a, uint32_t b) { return __umulhi(a, b); }
 __device__ __forceinline__ uint64_t mulhi(uint64_t a, uint64_t b) { return __umul64hi(a, b); }
 
