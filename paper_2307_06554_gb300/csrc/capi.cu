@@ -90,6 +90,26 @@ int upload_ntt_tables(polymul_plan* p) {
   return POLYMUL_OK;
 }
 
+// Tables of the unit for the smallest moduli (ntt_tiny.cuh).
+int upload_tiny_tables(polymul_plan* p) {
+  std::vector<uint32_t> all_f, all_i, f, i;
+  std::vector<PrimeConst<uint32_t>> pcs(p->k);
+  for (uint32_t j = 0; j < p->k; ++j) {
+    build_tiny_tables(p->q[j], p->n, f, i, pcs[j], p->cyclic);
+    all_f.insert(all_f.end(), f.begin(), f.end());
+    all_i.insert(all_i.end(), i.begin(), i.end());
+  }
+  auto up = [](void** dst, const void* src, size_t bytes) -> int {
+    PM_CUDA(cudaMalloc(dst, bytes));
+    PM_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
+    return POLYMUL_OK;
+  };
+  int r = up(&p->d_tiny_f, all_f.data(), all_f.size() * sizeof(uint32_t));
+  if (r == POLYMUL_OK) r = up(&p->d_tiny_i, all_i.data(), all_i.size() * sizeof(uint32_t));
+  if (r == POLYMUL_OK) r = up(&p->d_tiny_pc, pcs.data(), pcs.size() * sizeof(pcs[0]));
+  return r;
+}
+
 // Auxiliary NTT prime for moduli without a 2n-th root of unity: the largest
 // prime p < 2^31 with 2n | p - 1; usable when p > 2 n floor(qmax/2)^2 (the
 // centred integer product then fits in (-p/2, p/2)).  0 if none.
@@ -475,7 +495,14 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     // the default kernel first, then the candidates the autotuner may prefer
     rc = p->elem == 4 ? upload_ntt_tables<uint32_t>(p) : upload_ntt_tables<uint64_t>(p);
     KernelInfo v;
-    if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, p->ki);
+    const KernelInfo word = p->ki;
+    // moduli below 18500 (12289 and the like), n = 2^8 .. 2^10: the unit of
+    // ntt_tiny.cuh first (see there for the bound and the measurements)
+    if (rc == POLYMUL_OK && p->elem == 4 && qmax < kTinyQMax && lookup_ntt_tiny((int)p->logn, &v)) {
+      rc = upload_tiny_tables(p);
+      if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, v);
+    }
+    if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, word);
     if (rc == POLYMUL_OK && p->elem == 4 && lookup_ntt_u32_rb5((int)p->logn, p->mode, &v) && v.fn != p->cands[0].ki.fn)
       rc = add_candidate(POLYMUL_PATH_NTT, v);
     if (rc == POLYMUL_OK && p->elem == 4 && p->logn == 14 &&
@@ -530,6 +557,9 @@ extern "C" void polymul_destroy(polymul_plan* p) {
   cudaFree(p->d_twf);
   cudaFree(p->d_twi);
   cudaFree(p->d_pc);
+  cudaFree(p->d_tiny_f);
+  cudaFree(p->d_tiny_i);
+  cudaFree(p->d_tiny_pc);
   cudaFree(p->d_tpc);
   cudaFree(p->d_tpc8);
   cudaFree(p->d_tp64);
@@ -700,6 +730,20 @@ static int validate_operands(polymul_plan* p, const void* a, const void* b, uint
   return POLYMUL_OK;
 }
 
+// The unit of the smallest moduli (eight warps per CTA): fewer warps per CTA
+// when the batch would leave SMs empty otherwise, so that it spreads over all
+// of them.
+static void cta_warps(const polymul_plan* p, uint64_t units, int* block, int* smem, int* units_per_cta) {
+  const int warps = *block / 32, per_warp = *units_per_cta / warps;
+  const uint64_t one_each = (uint64_t)per_warp * p->num_sms;  // units of one warp on every SM
+  const uint64_t want = (units + one_each - 1) / one_each;
+  if (want >= (uint64_t)warps) return;
+  const int w = (int)std::max<uint64_t>(1, want);
+  *smem = *smem / warps * w;
+  *block = 32 * w;
+  *units_per_cta = per_warp * w;
+}
+
 int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_t batch, cudaStream_t st, int slot) {
   const uint64_t units = batch * p->k;
   unsigned long long* ctr = p->d_ctr + 2 * slot;
@@ -707,7 +751,9 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     const int r = validate_operands(p, a, b, units, st);
     if (r != POLYMUL_OK) return r;
   }
-  const uint64_t need = (units + p->ki.units_per_cta - 1) / p->ki.units_per_cta;
+  int block = p->ki.block, smem = p->ki.smem, units_per_cta = p->ki.units_per_cta;
+  if (p->ki.tiny) cta_warps(p, units, &block, &smem, &units_per_cta);
+  const uint64_t need = (units + units_per_cta - 1) / units_per_cta;
   int grid = (int)std::min<uint64_t>(need, (uint64_t)p->grid_cap);
   if (p->ki.cluster > 0) {
     const uint64_t clusters = std::min<uint64_t>(units, (uint64_t)(p->grid_cap / p->ki.cluster));
@@ -736,8 +782,8 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
       attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr.val.programmaticStreamSerializationAllowed = 1;
       cfg.gridDim = dim3(grid);
-      cfg.blockDim = dim3(p->ki.block);
-      cfg.dynamicSmemBytes = p->ki.smem;
+      cfg.blockDim = dim3(block);
+      cfg.dynamicSmemBytes = smem;
       cfg.stream = st;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
@@ -816,9 +862,13 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     uint32_t tx_pad = 0, polls = 0;
     if (p->ki.cluster == 0) take_injected_wait(&tx_pad, &polls);  // the cluster kernel has no copy waits
     if (p->elem == 4) {
-      NttBatchArgs<uint32_t> args{(const uint32_t*)a, (const uint32_t*)b, (uint32_t*)c, p->d_twf, p->d_twi,
-                                  (const PrimeConst<uint32_t>*)p->d_pc, units, p->k, ctr, p->d_err,
-                                  (const uint32_t*)p->d_outer, nullptr, p->n, 1, 0, early, tx_pad, polls};
+      const bool tiny = p->ki.tiny != 0;
+      // table strides count pairs of words; the tiny tables have n / 8 words per prime
+      NttBatchArgs<uint32_t> args{(const uint32_t*)a, (const uint32_t*)b, (uint32_t*)c,
+                                  tiny ? p->d_tiny_f : p->d_twf, tiny ? p->d_tiny_i : p->d_twi,
+                                  (const PrimeConst<uint32_t>*)(tiny ? p->d_tiny_pc : p->d_pc), units, p->k, ctr,
+                                  p->d_err, (const uint32_t*)p->d_outer, nullptr, tiny ? p->n / 16 : p->n, 1, 0, early,
+                                  tx_pad, polls};
       void* argv[] = {&args};
       r = launch(argv);
     } else {

@@ -18,6 +18,7 @@ struct KernelInfo {
   int regs = 0;              // NTT: register budget per thread
   int pad = 0;               // NTT: exchange layout (0 XOR swizzle, s > 0 one padding word per 2^s)
   int seq = 0;               // NTT: 1 = one operand in registers at a time
+  int tiny = 0;              // NTT: 1 = the unit for the smallest moduli (ntt_tiny.cuh), with its own tables
   int tiled = 0;             // tensor path: 1 for k_toeplitz_tiled (output groups, K chunks)
   int drain = 0;             // tensor path: tiled kernel draining each K chunk (8-bit digits at any n)
   int ws = 0;                // tensor path: the drained kernel's warp-specialised pipeline (k_toeplitz_ws)
@@ -33,6 +34,7 @@ bool lookup_ntt_u32_m1(int logn, KernelInfo* ki);
 bool lookup_ntt_u32_m2(int logn, KernelInfo* ki);
 bool lookup_ntt_u64_m1(int logn, KernelInfo* ki);  // logn 4..13
 bool lookup_ntt_u64_m2(int logn, KernelInfo* ki);
+bool lookup_ntt_tiny(int logn, KernelInfo* ki);     // moduli below 18500, logn 8..10
 bool lookup_ntt_u32_aux(int logn, KernelInfo* ki);  // auxiliary-prime mode, logn 4..14
 bool lookup_ntt_u32_aux_rb2(int logn, KernelInfo* ki);  // the same with radix-4 passes, logn 7..10
 // autotuner candidates: other register radices (RB = stage bits per pass)

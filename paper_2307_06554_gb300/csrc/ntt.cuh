@@ -134,8 +134,10 @@ __device__ __forceinline__ uint32_t xpos(uint32_t j) {
 //          conditional subtraction anywhere.  Forward values grow by at most
 //          2q per stage ((1+2s)q after s stages); inverse values at most
 //          double per stage (2^(s+1) q after s stages), the subtraction
-//          offset of stage s being that bound.
-enum { kQ31 = 0, kL4 = 1, kSmall = 2 };
+//          offset of stage s being that bound;
+//   kTiny  q < 18500, n = 2^8 .. 2^10: the unit of ntt_tiny.cuh (signed
+//          residues, its own tables).
+enum { kQ31 = 0, kL4 = 1, kSmall = 2, kTiny = 3 };
 
 template <typename W, int MODE>
 __device__ __forceinline__ void ct_bfly(W& x, W& y, const TwPair<W>& w, const PrimeConst<W>& pc) {
@@ -577,7 +579,7 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
     sa[e * S::T + t] = x[e];
   });
   load_top(ib);
-  fwd_from1<S, MODE, TOP>(x, sb, twf, pc, t, sync);
+  fwd_from1<S, MODE, TOP>(x, sb, twf + pc.zero, pc, t, sync);
   sfor<0, S::R>([&](auto ec) {
     constexpr int e = decltype(ec)::value;
     const W y = sa[e * S::T + t];
@@ -611,12 +613,19 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
   }
 }
 
+}  // namespace pm
+#include "ntt_tiny.cuh"
+namespace pm {
+
 template <class S, int MODE, bool AUX, bool SEQ, class Sync, class Hook, typename W = typename S::W>
 __device__ __forceinline__ void polymul_unit_any(W* __restrict__ c, const TwPair<W>* __restrict__ twf,
                                                  const TwPair<W>* __restrict__ twi, const PrimeConst<W>& pc,
                                                  W* sa, W* sb, const W* ia, const W* ib, uint32_t t, bool act,
                                                  Sync sync, Hook&& hook, W qo = 0) {
-  if constexpr (SEQ)
+  if constexpr (MODE == kTiny)
+    polymul_unit_tiny<S>(c, reinterpret_cast<const int*>(twf), reinterpret_cast<const int*>(twi), pc, sa, sb, ia, ib, t,
+                         act, sync, hook);
+  else if constexpr (SEQ)
     polymul_unit_seq<S, MODE, AUX>(c, twf, twi, pc, sa, sb, ia, ib, t, act, sync, hook, qo);
   else
     polymul_unit<S, MODE, AUX>(c, twf, twi, pc, sa, sb, ia, ib, t, act, sync, hook, qo);
@@ -705,7 +714,10 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     if (lane == 0) mbar_init(bar, 1);
     fence_mbar_init();
     __syncwarp();
-    const unsigned long long first_round = (unsigned long long)gridDim.x * WARPS * TPW;
+    // warps of this launch's CTAs: at most WARPS, fewer where the batch would
+    // not fill the SMs (see cta_warps in capi.cu)
+    const uint32_t warps = blockDim.x >> 5;
+    const unsigned long long first_round = (unsigned long long)gridDim.x * warps * TPW;
     auto grab = [&]() {  // every lane of the warp
       order();
       unsigned long long v = 0;
@@ -725,7 +737,7 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     uint32_t parity = 0;
     // first units by position (no atomic on the critical path at start-up),
     // later ones from the counter, offset by the units handed out that way
-    unsigned long long cur = ((unsigned long long)blockIdx.x * WARPS + warp) * TPW;
+    unsigned long long cur = ((unsigned long long)blockIdx.x * warps + warp) * TPW;
     if (!DIRECT && lane == 0 && cur < units) issue(cur);
     while (cur < units) {
       if constexpr (!DIRECT) {
@@ -764,7 +776,7 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     // kernel's completion, and every grab above returned before its team
     // got here
     if (lane == 0) {
-      const unsigned long long teams = (unsigned long long)gridDim.x * WARPS;
+      const unsigned long long teams = (unsigned long long)gridDim.x * warps;
       if (atomicAdd(ctr + 1, 1ull) == teams - 1) {
         atomicExch(ctr, 0ull);
         atomicExch(ctr + 1, 0ull);

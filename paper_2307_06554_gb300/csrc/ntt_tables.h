@@ -50,7 +50,7 @@ inline void build_ntt_tables_into(uint64_t q, uint32_t n, W* twf, W* twi, PrimeC
   pc.scale_p = (W)shoup_companion(scale, q, bits);
   pc.scale_w = (W)scale_w;
   pc.scale_wp = (W)shoup_companion(scale_w, q, bits);
-  pc.pad = 0;
+  pc.zero = 0;
 }
 
 template <typename W>
@@ -59,6 +59,45 @@ inline void build_ntt_tables(uint64_t q, uint32_t n, std::vector<W>& twf, std::v
   twf.resize(2 * (size_t)n);
   twi.resize(2 * (size_t)n);
   build_ntt_tables_into<W>(q, n, twf.data(), twi.data(), pc, cyclic);
+}
+
+// Tables of the unit for the smallest moduli (ntt_tiny.cuh): n / 8 words
+// forward and n / 8 inverse (entry k as in build_ntt_tables_into, k < n / 8;
+// the transform stops at polynomials of 8 coefficients, so a root of order
+// 2n / 8, n / 8 for the cyclic ring, is enough), each the word
+// (-w 2^32 mod q, centred) q^-1 mod 2^32 of a root w, and the constants the
+// unit reads from PrimeConst.
+constexpr uint32_t kTinyQMax = 18500;  // exclusive
+inline uint32_t tiny_word(uint64_t w, uint64_t q) {
+  const int64_t W = (int64_t)((q - w % q * ((1ull << 32) % q) % q) % q);
+  const int64_t centred = W > (int64_t)(q / 2) ? W - (int64_t)q : W;
+  return (uint32_t)((uint64_t)centred * pm::host::inv_pow2_64(q));
+}
+inline void build_tiny_tables(uint64_t q, uint32_t n, std::vector<uint32_t>& twf, std::vector<uint32_t>& twi,
+                              PrimeConst<uint32_t>& pc, bool cyclic = false) {
+  using namespace pm::host;
+  const uint32_t m = n / 8;
+  const int logm = __builtin_ctz(m);
+  const uint64_t psi = cyclic ? primitive_n_root(q, m) : primitive_2n_root(q, m);
+  const uint64_t psi_inv = powmod(psi, q - 2, q);
+  twf.assign(m, 0);
+  twi.assign(m, 0);
+  for (uint32_t i = 1; i < m; ++i) {
+    const uint32_t r = cyclic ? bitrev(i - (1u << (31 - __builtin_clz(i))), logm) / 2 : bitrev(i, logm);
+    twf[i] = tiny_word(powmod(psi, r, q), q);
+    twi[i] = tiny_word(powmod(psi_inv, r, q), q);
+  }
+  // the products of the small rings come out times -2^-32
+  const uint64_t r32 = (1ull << 32) % q;
+  const uint64_t scale = mulmod(powmod(m, q - 2, q), (q - r32) % q, q);
+  const uint64_t v1 = cyclic ? 1 : powmod(psi_inv, bitrev(1, logm), q);
+  pc = PrimeConst<uint32_t>{};
+  pc.q = (uint32_t)q;
+  pc.q2 = (uint32_t)(2 * q);
+  pc.qinv = (uint32_t)inv_pow2_64(q);
+  pc.scale = tiny_word(scale, q);
+  pc.scale_p = tiny_word(1, q);
+  pc.scale_w = tiny_word(mulmod(v1, scale, q), q);
 }
 
 // Reduction mode for the largest modulus (see the mode notes in ntt.cuh):

@@ -39,6 +39,10 @@ struct polymul_plan {
   void* d_twf = nullptr;
   void* d_twi = nullptr;
   void* d_pc = nullptr;
+  // the same for the unit of the smallest moduli, when a candidate uses it
+  void* d_tiny_f = nullptr;
+  void* d_tiny_i = nullptr;
+  void* d_tiny_pc = nullptr;
   pm::KernelInfo ki;   // the main kernel of the chosen path
   pm::KernelInfo tki;  // tensor-path kernel, when one exists for the shape
   std::vector<PlanCandidate> cands;  // [0] is the default

@@ -14,7 +14,7 @@ struct alignas(16) PrimeConst {
   W scale_p;   // Shoup companion of scale
   W scale_w;   // psi^-brv(1) * scale mod q (last inverse stage twiddle)
   W scale_wp;  // Shoup companion of scale_w
-  W pad;
+  W zero;      // 0, as a value the compiler cannot know (see polymul_unit_seq)
 };
 
 // One (product, prime) row of an uneven list: its element offset in a, b, c

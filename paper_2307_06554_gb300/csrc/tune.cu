@@ -60,6 +60,7 @@ void store_cache(const std::string& key, const std::string& label) {
 
 std::string label_of(const PlanCandidate& c) {
   if (c.path == POLYMUL_PATH_TENSOR) return c.ki.rns ? "tensor-rns" : c.ki.tiled ? "tensor-tiled" : "tensor";
+  if (c.ki.tiny) return "ntt-tiny";
   return "ntt-rb" + std::to_string(c.ki.rb) + (c.ki.cluster ? "-cluster" : "");
 }
 
@@ -89,7 +90,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
   const size_t prod_bytes = (size_t)p->k * p->n * p->elem;
   while (bucket > 1 && 3 * bucket * prod_bytes > (1ull << 30)) bucket >>= 1;  // at most 1 GiB of scratch
   char keybuf[256];
-  snprintf(keybuf, sizeof keybuf, "%s|w%u|n%u|k%u|m%d|q%d|b%llu", prop.name, p->elem, p->n, p->k, p->mode, qbits,
+  snprintf(keybuf, sizeof keybuf, "%s|w%u|n%u|k%u|m%d|q%d|b%llu", prop.name, p->elem, p->n, p->k, p->d_tiny_f ? 3 : p->mode, qbits,
            (unsigned long long)bucket);
   const std::string key(keybuf);
   std::lock_guard<std::mutex> lock(g_tune_mu);
