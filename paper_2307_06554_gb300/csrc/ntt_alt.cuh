@@ -1,6 +1,6 @@
 // Alternative k_ntt_batch shapes per degree (see NttCfg in ntt_info.cuh):
-// where the default is padded, the swizzled two-operand kernel at 128
-// registers; where it is swizzled, the padded one-operand kernel at 96.
+// the swizzled two-operand kernel at 128 registers up to 2^11, the padded
+// one-operand kernel at 96 above.
 #pragma once
 #include "ntt_info.cuh"
 

@@ -1,8 +1,6 @@
 // k_ntt_batch alternative shapes, 64-bit words, reduction mode 1 (autotuner
 // candidates): radix 16, padded, both operands, 128 registers where the
-// default is the radix-8 one-operand kernel (2^6 .. 2^11), and that radix-8
-// kernel where the default is radix 16 (2^12; at 2^13 its 1024-thread CTA
-// leaves 64 registers per thread).
+// default is a radix-8 kernel (2^6 .. 2^12).
 #include "ntt_alt.cuh"
 
 namespace pm {
@@ -22,14 +20,8 @@ bool lookup_ntt_alt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
   case L:                                                           \
     *ki = ntt_info_x<uint64_t, L, 1, false, 4, 128, 4, false>();    \
     return true;
-#define PM_R8(L)                                                    \
-  case L:                                                           \
-    *ki = ntt_info_x<uint64_t, L, 1, false, 3, 96, 3, true>();      \
-    return true;
-    PM_R16(6) PM_R16(7) PM_R16(8) PM_R16(9) PM_R16(10) PM_R16(11)
-    PM_R8(12)
+    PM_R16(6) PM_R16(7) PM_R16(8) PM_R16(9) PM_R16(10) PM_R16(11) PM_R16(12)
 #undef PM_R16
-#undef PM_R8
     default:
       return false;
   }

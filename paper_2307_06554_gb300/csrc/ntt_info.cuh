@@ -11,23 +11,44 @@ constexpr int kNttWarps = 4;  // warps per CTA when a team fits in a warp
 // register pass (RB), exchange layout (PAD: 0 the XOR swizzle, else the
 // padded layout with one word after every 2^PAD), register budget per thread
 // and whether one operand at a time is held in registers (SEQ).  Measured on
-// GB300 with 2^22 coefficients per batch (2^21 for 64-bit words), reduction
-// modes 1 and 2, launches back to back:
-//   32-bit words, n <= 2^9:      radix 16, padded, 96 registers, both operands;
-//   32-bit words, n = 2^10,2^11: radix 16, padded, 96 registers, one operand
-//                                 (n = 1024, q = 12289: 27.0 -> 25.7 us);
-//   32-bit words, n >= 2^12:     radix 16, swizzled, 128 registers (the
-//                                 padded kernels were 5-10 % slower there);
+// GB300 with 2^22 coefficients per batch (2^21 for 64-bit words), launches
+// back to back:
+//   32-bit words, n <= 2^11:     radix 16, padded, 96 registers, both operands
+//                                 (one operand at a time at 2^10, 2^11: 29.7
+//                                 and 32.5 us against 28.5 and 30.3 for 4 M
+//                                 coefficients, q < 2^30; 64 registers win only
+//                                 beyond 16 M), except
+//   ... unreduced mode, 2^10, 2^11: one operand (n = 1024, q = 12289: 27.0 ->
+//                                 25.7 us);
+//   32-bit words, n >= 2^12:     radix 16, padded, 64 registers, both operands:
+//                                 32 warps per SM hold the multiply pipe at
+//                                 74 % of its cycles.  16 M coefficients,
+//                                 q < 2^31: 112.4 us at 2^12 (swizzled, 128
+//                                 registers: 123.0), 141.3 at 2^13 (164.6);
+//                                 8 M, q < 2^30, 2^12: 57.2 (62.0).  2^14 takes
+//                                 a 512-thread CTA of its own (ntt_u32_rb5.cu);
 //   64-bit words, 2^6 .. 2^11:   radix 8, padded, 96 registers, one operand
 //                                 (radix 16 spills: 1.35-1.47x faster);
-//   64-bit words, 2^12, 2^13:    radix 16, padded, 128 registers.
-template <typename W, int LOGN>
+//   64-bit words, 2^12:          radix 8, padded, 64 registers, both operands:
+//                                 twice the threads per unit and half the
+//                                 straight-line code of radix 16, whose fetch
+//                                 stalled it (n = 4096: 152 units 26.9 -> 20.3
+//                                 us, 608 units 82.1 -> 67.2, 2048 units 233 ->
+//                                 227; at 2^11 and 2^10 the spills of its 64
+//                                 registers outweigh that).  The
+//                                 multiply pipe then bounds it (65 % of its
+//                                 cycles; loops over the passes in place of the
+//                                 straight line cut the fetch stalls to nothing
+//                                 and gained nothing more);
+//   64-bit words, 2^13:          radix 16, padded, 128 registers (radix 8 with
+//                                 1024 threads: the same time).
+template <typename W, int LOGN, int MODE = 1>
 struct NttCfg {
   static constexpr bool u32 = sizeof(W) == 4;
-  static constexpr int RB = u32 ? 4 : (LOGN >= 6 && LOGN <= 11 ? 3 : 4);
-  static constexpr int PAD = u32 ? (LOGN >= 5 && LOGN <= 11 ? 4 : 0) : (LOGN >= 6 ? RB : 0);
-  static constexpr int REGS = u32 ? (LOGN >= 5 && LOGN <= 11 ? 96 : 128) : (LOGN >= 6 && LOGN <= 11 ? 96 : 128);
-  static constexpr bool SEQ = u32 ? (LOGN == 10 || LOGN == 11) : (LOGN >= 6 && LOGN <= 11);
+  static constexpr int RB = u32 ? 4 : (LOGN >= 6 && LOGN <= 12 ? 3 : 4);
+  static constexpr bool SEQ = u32 ? MODE == kSmall && (LOGN == 10 || LOGN == 11) : (LOGN >= 6 && LOGN <= 11);
+  static constexpr int PAD = u32 ? (LOGN >= 5 ? 4 : 0) : (LOGN >= 6 ? RB : 0);
+  static constexpr int REGS = u32 ? (LOGN < 5 ? 128 : LOGN < 12 ? 96 : 64) : (LOGN >= 6 && LOGN <= 11 ? 96 : LOGN == 12 ? 64 : 128);
 };
 
 // every parameter explicit
@@ -56,7 +77,7 @@ KernelInfo ntt_info_x() {
 // the default shape for (W, LOGN)
 template <typename W, int LOGN, int MODE, bool AUX = false>
 KernelInfo ntt_info() {
-  using C = NttCfg<W, LOGN>;
+  using C = NttCfg<W, LOGN, MODE>;
   return ntt_info_x<W, LOGN, MODE, AUX, C::RB, C::REGS, C::PAD, C::SEQ>();
 }
 
