@@ -316,10 +316,9 @@ bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
     // beyond one CTA: one product per thread-block cluster, the form with
     // CTA-local exchanges (measured on GB300 against the first form: 64-bit
     // words with both operands in registers 1.38-1.49x faster at 2^14 ..
-    // 2^16; 32-bit words one operand at a time 1.2x at 2^15, 2^16); the
-    // unreduced mode takes the Harvey-bound kernels, whose bounds hold for
-    // its moduli too
-    if (lookup_ntt_cluster2(elem, logn, mode == 2 ? 1 : mode, elem == 4, ki)) return true;
+    // 2^16; 32-bit words see lookup_ntt_cluster2); the unreduced mode takes
+    // the Harvey-bound kernels, whose bounds hold for its moduli too
+    if (lookup_ntt_cluster2(elem, logn, mode == 2 ? 1 : mode, false, ki)) return true;
     return lookup_ntt_cluster(elem, logn, mode, ki) || (mode == 2 && lookup_ntt_cluster(elem, logn, 1, ki));
   }
   if (elem == 4) {
@@ -354,11 +353,28 @@ int pm::tmem_kernel_per_sm(const KernelInfo& ki, int device, int* per_sm) {
 
 namespace {
 
+// 32-bit batch kernels with one product per CTA of 256 or 512 threads (n =
+// 2^12, 2^13) hold four or two CTAs per SM.  A batch with fewer units than
+// that asks for enough shared memory that each SM takes its share of them and
+// no more: launches start while the previous one still runs, and its leftover
+// slots are spread unevenly (125 products at 2^13, overlapped batches: 15.9
+// us per batch unlimited, 11.1 with one CTA per SM).
+bool spread_launch(const polymul_plan* p, const KernelInfo& ki) {
+  return p->elem == 4 && ki.cluster == 0 && ki.tmem_cols == 0 && (ki.team == 256 || ki.team == 512);
+}
+// dynamic shared memory with which exactly `per_sm` CTAs fit on an SM
+int spread_smem(const polymul_plan* p, int per_sm) {
+  return (p->smem_sm / (per_sm + 1) - p->smem_resv + 15) / 16 * 16 + 16;
+}
+
 int configure_launch(polymul_plan* p) {
   PM_CUDA(cudaGetDevice(&p->device));
   PM_CUDA(cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device));
-  if (p->ki.smem > 48 * 1024)
-    PM_CUDA(cudaFuncSetAttribute(p->ki.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->ki.smem));
+  PM_CUDA(cudaDeviceGetAttribute(&p->smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, p->device));
+  PM_CUDA(cudaDeviceGetAttribute(&p->smem_resv, cudaDevAttrReservedSharedMemoryPerBlock, p->device));
+  const int smem_max = spread_launch(p, p->ki) ? std::max(p->ki.smem, spread_smem(p, 1)) : p->ki.smem;
+  if (smem_max > 48 * 1024)
+    PM_CUDA(cudaFuncSetAttribute(p->ki.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max));
   PM_CUDA(cudaFuncSetAttribute(p->ki.fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
   int per_sm = 0;
   if (p->ki.cluster > 0) {
@@ -464,6 +480,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   };
 
   int rc = POLYMUL_OK;
+  size_t few = 0;  // the candidate for few products, if there is one
   // NTT batch kernels take a programmatic dependent launch (measured on
   // back-to-back batches: n = 1024, 4096 products 29.9 -> 27.6 us; n = 256,
   // 64 products 8.3 -> 5.7 us); cluster and tensor kernels take plain launches
@@ -520,11 +537,57 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
           (lookup_ntt_cluster(p->elem, (int)p->logn, p->mode, &v) || lookup_ntt_cluster(p->elem, (int)p->logn, 1, &v)))
         rc = add_candidate(POLYMUL_PATH_NTT, v);
     }
-    if (rc == POLYMUL_OK && p->elem == 4 && lookup_ntt_u32_rb3((int)p->logn, p->mode, &v)) rc = add_candidate(POLYMUL_PATH_NTT, v);
-    if (rc == POLYMUL_OK && p->logn < 14 && lookup_ntt_alt(p->elem, (int)p->logn, p->mode, &v)) rc = add_candidate(POLYMUL_PATH_NTT, v);
+    if (rc == POLYMUL_OK && p->elem == 4 && lookup_ntt_u32_rb3((int)p->logn, p->mode, &v)) {
+      rc = add_candidate(POLYMUL_PATH_NTT, v);
+      // radix 8, twice the threads per product (30-bit primes, n = 1024: 8
+      // products 4.6 us against 5.3, 304 products 5.4 / 5.9, 608 products the
+      // same; n = 2048: 152 products 5.9 / 6.4, 304 products the same)
+      if (p->logn <= 11) few = p->cands.size() - 1;
+    }
+    if (rc == POLYMUL_OK && p->logn < 14 && lookup_ntt_alt(p->elem, (int)p->logn, p->mode, &v)) {
+      rc = add_candidate(POLYMUL_PATH_NTT, v);
+      // 32-bit words, n = 2^13, one product per SM at most: nothing else runs
+      // beside it, and 128 registers hold more loads in flight (125 products,
+      // q < 2^20: 12.7 us against 13.3)
+      if (p->elem == 4 && p->logn == 13) few = p->cands.size() - 1;
+    }
+    // n >= 2^13 (64-bit words), 2^14 (32-bit): few products over more CTAs
+    // each, up to the number at which that no longer pays.  64-bit words: at
+    // 2^15 8 products 30.7 us against 49.1 and 30 products 52.1 / 50.2; at
+    // 2^14 24 products 28.8 / 45.2, 38 products the same; at 2^13 64 products
+    // 26.6 / 40.6, 111 products 43.1 / 41.0.  32-bit words at 2^14: 64
+    // products 18.7 / 25.3, 111 products 28.2 / 25.7.
+    if (rc == POLYMUL_OK && p->logn >= (p->elem == 8 ? 13u : 14u) &&
+        lookup_ntt_cluster_small(p->elem, (int)p->logn, p->mode == 2 ? 1 : p->mode, &v)) {
+      rc = add_candidate(POLYMUL_PATH_NTT, v);
+      few = p->cands.size() - 1;
+    }
     if (rc == POLYMUL_OK && path == POLYMUL_PATH_AUTO && tensor_ok) rc = add_tensor_candidates(add_candidate);
   }
   if (rc == POLYMUL_OK) apply_candidate(p, 0);
+  if (rc == POLYMUL_OK && few) {
+    p->small = few;
+    const uint64_t sms = (uint64_t)p->num_sms;
+    if (p->elem == 8)
+      p->small_units = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
+    else
+      p->small_units = p->logn == 14 ? sms / 2 : p->logn == 13 ? sms : sms * 2048 / p->n;
+  }
+  // Small batches leave most of the GPU idle whatever the kernel: one unit's
+  // latency is the call, and more threads per unit with shorter chains win.
+  // Auxiliary-prime plans: the radix-4 kernel (n = 256, 64 units: 4.3 us
+  // against 6.8; 1024: 5.1 / 8.1) up to 3500 coefficients per SM, where the
+  // two meet (n = 512, 1216 units: 8.9 / 8.4).  Smallest moduli: the radix-16
+  // kernel (n = 1024, 64 units: 5.4 us against 6.9; n = 256, 152 units:
+  // 5.0 / 6.5) up to 4500 per SM (n = 1024, 608 units 7.5 / 7.5, 912 units
+  // 12.1 / 7.7; n = 256, 2432 units 6.3 / 7.5, 4864 units 9.7 / 7.6).
+  if (rc == POLYMUL_OK && p->cands.size() > 1) {
+    const bool aux2 = p->aux_prime != 0;
+    if (aux2 || p->cands[0].ki.tiny) {
+      p->small = 1;
+      p->small_units = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
+    }
+  }
   if (rc == POLYMUL_OK) {
     // work counters for the three launch slots (device entry, two host-entry streams)
     if (cudaMalloc(&p->d_ctr, 2 * kCounterSlots * sizeof(unsigned long long)) != cudaSuccess ||
@@ -730,20 +793,6 @@ static int validate_operands(polymul_plan* p, const void* a, const void* b, uint
   return POLYMUL_OK;
 }
 
-// The unit of the smallest moduli (eight warps per CTA): fewer warps per CTA
-// when the batch would leave SMs empty otherwise, so that it spreads over all
-// of them.
-static void cta_warps(const polymul_plan* p, uint64_t units, int* block, int* smem, int* units_per_cta) {
-  const int warps = *block / 32, per_warp = *units_per_cta / warps;
-  const uint64_t one_each = (uint64_t)per_warp * p->num_sms;  // units of one warp on every SM
-  const uint64_t want = (units + one_each - 1) / one_each;
-  if (want >= (uint64_t)warps) return;
-  const int w = (int)std::max<uint64_t>(1, want);
-  *smem = *smem / warps * w;
-  *block = 32 * w;
-  *units_per_cta = per_warp * w;
-}
-
 int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_t batch, cudaStream_t st, int slot) {
   const uint64_t units = batch * p->k;
   unsigned long long* ctr = p->d_ctr + 2 * slot;
@@ -751,30 +800,40 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     const int r = validate_operands(p, a, b, units, st);
     if (r != POLYMUL_OK) return r;
   }
-  int block = p->ki.block, smem = p->ki.smem, units_per_cta = p->ki.units_per_cta;
-  if (p->ki.tiny) cta_warps(p, units, &block, &smem, &units_per_cta);
-  const uint64_t need = (units + units_per_cta - 1) / units_per_cta;
-  int grid = (int)std::min<uint64_t>(need, (uint64_t)p->grid_cap);
-  if (p->ki.cluster > 0) {
-    const uint64_t clusters = std::min<uint64_t>(units, (uint64_t)(p->grid_cap / p->ki.cluster));
-    grid = (int)(clusters * p->ki.cluster);
+  // the kernel: the plan's choice, or the candidate for batches this small
+  // (a pending diagnostics injection counts launches of the batch kernel, so
+  // it keeps the plan's choice)
+  const PlanCandidate* small =
+      units <= p->small_units && !injected_wait_pending() ? &p->cands[p->small] : nullptr;
+  const KernelInfo& ki = small ? small->ki : p->ki;
+  const int grid_cap = small ? small->grid_cap : p->grid_cap;
+  const uint64_t need = (units + ki.units_per_cta - 1) / ki.units_per_cta;
+  int grid = (int)std::min<uint64_t>(need, (uint64_t)grid_cap);
+  int smem = ki.smem;
+  if (spread_launch(p, ki)) {
+    const int per_sm = (grid + p->num_sms - 1) / p->num_sms;
+    if (per_sm < grid_cap / p->num_sms) smem = std::max(smem, spread_smem(p, per_sm));
+  }
+  if (ki.cluster > 0) {
+    const uint64_t clusters = std::min<uint64_t>(units, (uint64_t)(grid_cap / ki.cluster));
+    grid = (int)(clusters * ki.cluster);
   }
   auto launch = [&](void** argv) -> int {
-    if (p->ki.cluster > 0) {
+    if (ki.cluster > 0) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof cfg);
       cudaLaunchAttribute attr;
       attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = p->ki.cluster;
+      attr.val.clusterDim.x = ki.cluster;
       attr.val.clusterDim.y = 1;
       attr.val.clusterDim.z = 1;
       cfg.gridDim = dim3(grid);
-      cfg.blockDim = dim3(p->ki.block);
-      cfg.dynamicSmemBytes = p->ki.smem;
+      cfg.blockDim = dim3(ki.block);
+      cfg.dynamicSmemBytes = ki.smem;
       cfg.stream = st;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      PM_CUDA(cudaLaunchKernelExC(&cfg, p->ki.fn, argv));
+      PM_CUDA(cudaLaunchKernelExC(&cfg, ki.fn, argv));
     } else if (p->launch_flags & kLaunchPdl) {
       cudaLaunchConfig_t cfg;
       memset(&cfg, 0, sizeof cfg);
@@ -782,18 +841,18 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
       attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
       attr.val.programmaticStreamSerializationAllowed = 1;
       cfg.gridDim = dim3(grid);
-      cfg.blockDim = dim3(block);
+      cfg.blockDim = dim3(ki.block);
       cfg.dynamicSmemBytes = smem;
       cfg.stream = st;
       cfg.attrs = &attr;
       cfg.numAttrs = 1;
-      PM_CUDA(cudaLaunchKernelExC(&cfg, p->ki.fn, argv));
+      PM_CUDA(cudaLaunchKernelExC(&cfg, ki.fn, argv));
     } else {
-      PM_CUDA(cudaLaunchKernel(p->ki.fn, grid, p->ki.block, argv, p->ki.smem, st));
+      PM_CUDA(cudaLaunchKernel(ki.fn, grid, ki.block, argv, ki.smem, st));
     }
     return POLYMUL_OK;
   };
-  if (p->path == POLYMUL_PATH_TENSOR && p->ki.rns) {
+  if (p->path == POLYMUL_PATH_TENSOR && ki.rns) {
     RnsCfg rc;
     if (!rns_config((int)p->logn, p->rns_r, &rc)) return fail(POLYMUL_ENOTSUP, "tensor RNS tiling");
     // residue planes of a and b (slot-private scratch), then the MMA kernel
@@ -813,39 +872,39 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
                        p->cyclic ? 0u : 0x80008000u, p->logn, rc.shifts, rc.nb, rc.b_pitch, rc.ngrp, rc.kc, rc.a_win,
                        rc.bt_off, rc.buf_bytes, rc.tmem_cols, ctr, p->d_err};
     void* argv[] = {&args};
-    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)p->grid_cap);
-    PM_CUDA(cudaLaunchKernel(p->ki.fn, tgrid, p->ki.block, argv, p->ki.smem, st));
-  } else if (p->path == POLYMUL_PATH_TENSOR && p->ki.u64) {
+    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)grid_cap);
+    PM_CUDA(cudaLaunchKernel(ki.fn, tgrid, ki.block, argv, ki.smem, st));
+  } else if (p->path == POLYMUL_PATH_TENSOR && ki.u64) {
     TiledCfg tc;
-    if (!toeplitz_u64_config((int)p->logn, p->ki.digits, &tc)) return fail(POLYMUL_ENOTSUP, "tensor tiling (64-bit)");
+    if (!toeplitz_u64_config((int)p->logn, ki.digits, &tc)) return fail(POLYMUL_ENOTSUP, "tensor tiling (64-bit)");
     const uint64_t tunits = units * tc.ngrp;
     TensorU64Args args{(const uint64_t*)a, (const uint64_t*)b, (uint64_t*)c, (const TensorPrime64*)p->d_tp64, nullptr,
                        tunits, p->k, p->cyclic ? 0u : 0x80008000u, p->logn, tc.ngrp, tc.kc, tc.a_win, tc.bt_off,
                        tc.tmem_cols, ctr, p->d_err};
     void* argv[] = {&args};
-    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)p->grid_cap);
-    PM_CUDA(cudaLaunchKernel(p->ki.fn, tgrid, p->ki.block, argv, p->ki.smem, st));
-  } else if (p->path == POLYMUL_PATH_TENSOR && p->ki.tiled) {
+    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)grid_cap);
+    PM_CUDA(cudaLaunchKernel(ki.fn, tgrid, ki.block, argv, ki.smem, st));
+  } else if (p->path == POLYMUL_PATH_TENSOR && ki.tiled) {
     TiledCfg tc;
-    const DigitShape ds = digit_shape(p, p->ki);
-    if (!tiled_config_of(p->ki, (int)p->logn, ds.la, ds.lb, &tc)) return fail(POLYMUL_ENOTSUP, "tensor tiling");
+    const DigitShape ds = digit_shape(p, ki);
+    if (!tiled_config_of(ki, (int)p->logn, ds.la, ds.lb, &tc)) return fail(POLYMUL_ENOTSUP, "tensor tiling");
     const uint64_t tunits = units * tc.ngrp;
     // ternary b: c = b * T(a) (the ring is commutative), b's single digit on the A side
     const void* xa = p->ternary_b ? b : a;
     const void* xb = p->ternary_b ? a : b;
-    const void* tpc = p->ki.drain && p->d_tpc8 ? p->d_tpc8 : p->d_tpc;
+    const void* tpc = ki.drain && p->d_tpc8 ? p->d_tpc8 : p->d_tpc;
     TensorTiledArgs args{(const uint32_t*)xa, (const uint32_t*)xb, (uint32_t*)c, (const TensorPrime*)tpc,
                          tunits, p->k, p->cyclic ? 0u : 0x80008000u, p->logn, (uint32_t)ds.wb,
                          tc.bpg, tc.ngrp, tc.kc, tc.a_win, tc.bt_off, tc.tmem_cols, ctr, p->d_err, nullptr,
                          tc.stage_bytes};
     void* argv[] = {&args};
-    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)p->grid_cap);
-    PM_CUDA(cudaLaunchKernel(p->ki.fn, tgrid, p->ki.block, argv, p->ki.smem, st));
+    const int tgrid = (int)std::min<uint64_t>(tunits, (uint64_t)grid_cap);
+    PM_CUDA(cudaLaunchKernel(ki.fn, tgrid, ki.block, argv, ki.smem, st));
   } else if (p->path == POLYMUL_PATH_TENSOR) {
     TensorBatchArgs args{(const uint32_t*)a, (const uint32_t*)b, (uint32_t*)c, (const TensorPrime*)p->d_tpc,
                          units, p->k, p->cyclic ? 0u : 0x80008000u, ctr, p->d_err};
     void* argv[] = {&args};
-    PM_CUDA(cudaLaunchKernel(p->ki.fn, grid, p->ki.block, argv, p->ki.smem, st));
+    PM_CUDA(cudaLaunchKernel(ki.fn, grid, ki.block, argv, ki.smem, st));
   } else {
     // the batch kernel: record its footprint for the next launch on this
     // stream, and let it run ahead of the previous one where that is safe
@@ -856,13 +915,13 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     fp.b_lo = (uintptr_t)b, fp.b_hi = (uintptr_t)b + bytes;
     fp.c_lo = (uintptr_t)c, fp.c_hi = (uintptr_t)c + bytes;
     StreamOrderGuard order(p->device, st);
-    const bool pdl = p->ki.cluster == 0 && (p->launch_flags & kLaunchPdl);
+    const bool pdl = ki.cluster == 0 && (p->launch_flags & kLaunchPdl);
     const uint32_t early = pdl && (p->flags & POLYMUL_FLAG_OVERLAP) && order.may_run_ahead(fp) ? 1u : 0u;
     int r;
     uint32_t tx_pad = 0, polls = 0;
-    if (p->ki.cluster == 0) take_injected_wait(&tx_pad, &polls);  // the cluster kernel has no copy waits
+    if (ki.cluster == 0) take_injected_wait(&tx_pad, &polls);  // the cluster kernel has no copy waits
     if (p->elem == 4) {
-      const bool tiny = p->ki.tiny != 0;
+      const bool tiny = ki.tiny != 0;
       // table strides count pairs of words; the tiny tables have n / 8 words per prime
       NttBatchArgs<uint32_t> args{(const uint32_t*)a, (const uint32_t*)b, (uint32_t*)c,
                                   tiny ? p->d_tiny_f : p->d_twf, tiny ? p->d_tiny_i : p->d_twi,

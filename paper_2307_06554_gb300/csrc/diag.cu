@@ -32,6 +32,8 @@ bool take_injected_wait(uint32_t* tx_pad, uint32_t* polls) {
   return true;
 }
 
+bool injected_wait_pending() { return g_inject_launches.load() > 0; }
+
 __global__ void k_wait_selftest(uint32_t polls, int* err) {
   __shared__ __align__(8) uint64_t bar;
   if (threadIdx.x == 0) mbar_init(&bar, 1);

@@ -56,11 +56,17 @@ bool lookup_ntt_direct_aux(int logn, KernelInfo* ki);  // auxiliary-prime mode, 
 // logn 10..13, modes 0..2)
 bool lookup_ntt_shared(int logn, int mode, KernelInfo* prep, KernelInfo* main);
 
+// the same for the smallest moduli (ntt_tiny.cuh) in one launch, logn 10
+bool lookup_ntt_tiny_shared(int logn, KernelInfo* ki);
+
 // one product per thread-block cluster (n = 2^14 .. 2^16)
 bool lookup_ntt_cluster(uint32_t elem, int logn, int mode, KernelInfo* ki);
 // its second form: CTA-local exchanges except the top phase's, padded
 // layout; one operand in registers at a time (seq) or both (mode 1 only)
 bool lookup_ntt_cluster2(uint32_t elem, int logn, int mode, bool seq, KernelInfo* ki);
+// the second form over more CTAs, for few products: 64-bit words n = 2^12 ..
+// 2^15 (mode 1), 32-bit words n = 2^14 (modes 0, 1)
+bool lookup_ntt_cluster_small(uint32_t elem, int logn, int mode, KernelInfo* ki);
 
 // uneven batches (32-bit words): one persistent kernel for the degrees
 // 2^10..2^13 and one for 2^14, in two shape sets (0: swizzled exchanges,

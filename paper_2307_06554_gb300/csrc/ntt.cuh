@@ -579,7 +579,7 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
     sa[e * S::T + t] = x[e];
   });
   load_top(ib);
-  fwd_from1<S, MODE, TOP>(x, sb, twf + pc.zero, pc, t, sync);
+  fwd_from1<S, MODE, TOP>(x, sb, twf, pc, t, sync);
   sfor<0, S::R>([&](auto ec) {
     constexpr int e = decltype(ec)::value;
     const W y = sa[e * S::T + t];
@@ -714,10 +714,7 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     if (lane == 0) mbar_init(bar, 1);
     fence_mbar_init();
     __syncwarp();
-    // warps of this launch's CTAs: at most WARPS, fewer where the batch would
-    // not fill the SMs (see cta_warps in capi.cu)
-    const uint32_t warps = blockDim.x >> 5;
-    const unsigned long long first_round = (unsigned long long)gridDim.x * warps * TPW;
+    const unsigned long long first_round = (unsigned long long)gridDim.x * WARPS * TPW;
     auto grab = [&]() {  // every lane of the warp
       order();
       unsigned long long v = 0;
@@ -737,7 +734,7 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     uint32_t parity = 0;
     // first units by position (no atomic on the critical path at start-up),
     // later ones from the counter, offset by the units handed out that way
-    unsigned long long cur = ((unsigned long long)blockIdx.x * warps + warp) * TPW;
+    unsigned long long cur = ((unsigned long long)blockIdx.x * WARPS + warp) * TPW;
     if (!DIRECT && lane == 0 && cur < units) issue(cur);
     while (cur < units) {
       if constexpr (!DIRECT) {
@@ -776,7 +773,7 @@ __global__ void __launch_bounds__(ntt_block<S, WARPS>(), 65536 / (ntt_block<S, W
     // kernel's completion, and every grab above returned before its team
     // got here
     if (lane == 0) {
-      const unsigned long long teams = (unsigned long long)gridDim.x * warps;
+      const unsigned long long teams = (unsigned long long)gridDim.x * WARPS;
       if (atomicAdd(ctr + 1, 1ull) == teams - 1) {
         atomicExch(ctr, 0ull);
         atomicExch(ctr + 1, 0ull);

@@ -162,19 +162,27 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster(NttBatchArgs
 
 // ---------------------------------------------------------------- local exchanges
 // Second form of the cluster kernel.  Coefficient j's home is cluster rank
-// j >> 13 (8192 per CTA and operand), local index j & 8191.  In every layout
-// but the top phase's, the team-thread bits that select the CTA (bits 9 and
-// up of t = rank * 512 + thread) sit at coefficient bits 13 and up: each
+// j >> LL (2^LL per CTA and operand), its local index the low LL bits.  In
+// every layout but the top phase's, the team-thread bits that select the CTA
+// (those above the CTA's threads) sit at coefficient bits LL and up: each
 // thread's coefficients live in its own CTA, and an exchange between two such
 // layouts runs through the CTA's own shared memory with a CTA barrier (a warp
 // barrier when the warps keep their coefficients).  Only the exchange into
 // or out of the top phase reaches the other CTAs (distributed shared memory)
 // and takes the cluster barrier.  Buffers use the padded layout on the local
 // index (word jl at jl + (jl >> PAD)).
+// ClusterShape: 2^LL coefficients per CTA and operand, CT threads per CTA.
+template <typename W, int LOGN, int RB, int PAD, int LL_>
+struct ClusterShape : Shape<W, LOGN, RB, PAD> {
+  static constexpr int LL = LL_;
+  static constexpr int CTLOG = LL_ - RB;
+  static constexpr int CT = 1 << CTLOG;
+  static constexpr int CTAS = 1 << (LOGN - LL_);
+};
 template <class S, int P>
 constexpr bool cta_local() {
-  for (int b = 9; (1 << b) < S::T; ++b)
-    if (tbit_pos<S, P>(b) != b + (kClusterLocalLog - 9)) return false;
+  for (int b = S::CTLOG; (1 << b) < S::T; ++b)
+    if (tbit_pos<S, P>(b) != b + (S::LL - S::CTLOG)) return false;
   return true;
 }
 
@@ -197,8 +205,8 @@ __host__ __device__ constexpr uint32_t elem_index_c(int e) {
 // in place at each exchange (one mapa per rank; volatile, so that the
 // compiler does not keep 64-bit remote addresses alive across the unit).
 template <class S, typename W>
-__device__ __forceinline__ void rank_bases(W* local, W* (&rb)[S::T / kClusterThreads]) {
-  sfor<0, S::T / kClusterThreads>([&](auto rc) {
+__device__ __forceinline__ void rank_bases(W* local, W* (&rb)[S::CTAS]) {
+  sfor<0, S::CTAS>([&](auto rc) {
     constexpr int r = decltype(rc)::value;
     asm volatile("mapa.u64 %0, %1, %2;" : "=l"(rb[r]) : "l"(local), "r"(r));
   });
@@ -210,7 +218,7 @@ __device__ __forceinline__ void rank_bases(W* local, W* (&rb)[S::T / kClusterThr
 // slot part, and the padded position is additive over it)
 template <class S, int P, typename W = typename S::W>
 __device__ __forceinline__ void cstore(const W (&x)[S::R], W* buf, uint32_t t) {
-  constexpr uint32_t M = (1u << kClusterLocalLog) - 1u;
+  constexpr uint32_t M = (1u << S::LL) - 1u;
   W* base = buf + lpos<S>(elem_index<S, P>(0, t) & M);
   if constexpr (cta_local<S, P>()) {
     sfor<0, S::R>([&](auto ec) {
@@ -218,19 +226,19 @@ __device__ __forceinline__ void cstore(const W (&x)[S::R], W* buf, uint32_t t) {
       base[lpos<S>(elem_index<S, P>(e, 0) & M)] = x[e];
     });
   } else {
-    W* rb[S::T / kClusterThreads];
+    W* rb[S::CTAS];
     rank_bases<S>(base, rb);
     sfor<0, S::R>([&](auto ec) {
       constexpr int e = decltype(ec)::value;
       constexpr uint32_t je = elem_index_c<S, P>(e);  // the home rank comes from the slot bits
-      rb[je >> kClusterLocalLog][lpos<S>(je & M)] = x[e];
+      rb[je >> S::LL][lpos<S>(je & M)] = x[e];
     });
   }
 }
 
 template <class S, int P, typename W = typename S::W>
 __device__ __forceinline__ void cload(W (&x)[S::R], W* buf, uint32_t t) {
-  constexpr uint32_t M = (1u << kClusterLocalLog) - 1u;
+  constexpr uint32_t M = (1u << S::LL) - 1u;
   W* base = buf + lpos<S>(elem_index<S, P>(0, t) & M);
   if constexpr (cta_local<S, P>()) {
     sfor<0, S::R>([&](auto ec) {
@@ -238,12 +246,12 @@ __device__ __forceinline__ void cload(W (&x)[S::R], W* buf, uint32_t t) {
       x[e] = base[lpos<S>(elem_index<S, P>(e, 0) & M)];
     });
   } else {
-    W* rb[S::T / kClusterThreads];
+    W* rb[S::CTAS];
     rank_bases<S>(base, rb);
     sfor<0, S::R>([&](auto ec) {
       constexpr int e = decltype(ec)::value;
       constexpr uint32_t je = elem_index_c<S, P>(e);
-      x[e] = rb[je >> kClusterLocalLog][lpos<S>(je & M)];
+      x[e] = rb[je >> S::LL][lpos<S>(je & M)];
     });
   }
 }
@@ -307,18 +315,18 @@ __device__ __forceinline__ W pointwise1(W x, W y, const PrimeConst<W>& pc) {
 // their own.  Both operands at once (SEQ false): the inverse runs on a's
 // buffer, whose last remote reads the next unit's remote stores would race,
 // so each unit ends with a cluster barrier.
-template <class S, int MODE, bool SEQ>
-__global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster2(NttBatchArgs<typename S::W> args) {
+template <class S, int MODE, bool SEQ, int REGS>
+__global__ void __launch_bounds__(S::CT, 65536 / (S::CT * REGS)) k_ntt_cluster2(NttBatchArgs<typename S::W> args) {
   using W = typename S::W;
-  static_assert(S::T % kClusterThreads == 0 && S::N == (S::T / kClusterThreads) << kClusterLocalLog,
-                "one CTA per 8192 coefficients");
+  static_assert(S::T == S::CTAS * S::CT, "one CTA per 2^LL coefficients");
   static_assert(S::PAD > 0, "padded local layout");
   static_assert(!cta_local<S, S::NPH - 1>(), "the top layout spans the cluster");
+  static_assert(cta_local<S, S::NPH - 2>(), "every other layout is local to a CTA (see cstore)");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr uint32_t L = (1u << kClusterLocalLog) + ((1u << kClusterLocalLog) >> S::PAD);
+  constexpr uint32_t L = (1u << S::LL) + ((1u << S::LL) >> S::PAD);
   W* sa = reinterpret_cast<W*>(smem_raw);
   W* sb = sa + L;
-  const uint32_t t = cluster_rank() * kClusterThreads + threadIdx.x;
+  const uint32_t t = cluster_rank() * S::CT + threadIdx.x;
   constexpr int TOP = S::NPH - 1;
   const TwPair<W>* twf = reinterpret_cast<const TwPair<W>*>(args.tw_fwd);
   const TwPair<W>* twi = reinterpret_cast<const TwPair<W>*>(args.tw_inv);
@@ -342,7 +350,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster2(NttBatchArg
       __syncthreads();  // this CTA's layout-0 reads of sa are done
       sfor<0, S::R>([&](auto ec) {
         constexpr int e = decltype(ec)::value;
-        sa[e * kClusterThreads + threadIdx.x] = xa[e];
+        sa[e * S::CT + threadIdx.x] = xa[e];
       });
       sfor<0, S::R>([&](auto ec) {
         constexpr int e = decltype(ec)::value;
@@ -355,7 +363,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster2(NttBatchArg
       cfwd<S, MODE, TOP, false>(xa, xa, sb, sb, tf_b, pc, t);
       sfor<0, S::R>([&](auto ec) {
         constexpr int e = decltype(ec)::value;
-        xa[e] = pointwise1<S, MODE>(sa[e * kClusterThreads + threadIdx.x], xa[e], pc);
+        xa[e] = pointwise1<S, MODE>(sa[e * S::CT + threadIdx.x], xa[e], pc);
       });
       cinv<S, MODE, 0>(xa, sb, ti, pc, t);
     } else {
@@ -383,20 +391,20 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster2(NttBatchArg
   ClusterSync{}();  // no CTA leaves while another may still address its shared memory
 }
 
-template <typename W, int LOGN, int MODE, bool SEQ>
+template <typename W, int LOGN, int MODE, bool SEQ, int RB = 4, int LL = kClusterLocalLog, int REGS = 128>
 static KernelInfo cluster2_info() {
-  using S = Shape<W, LOGN, 4, 4>;
+  using S = ClusterShape<W, LOGN, RB, RB, LL>;
   KernelInfo ki;
-  ki.fn = (const void*)k_ntt_cluster2<S, MODE, SEQ>;
-  ki.block = kClusterThreads;
-  ki.smem = 2 * ((1 << kClusterLocalLog) + ((1 << kClusterLocalLog) >> 4)) * (int)sizeof(W);
+  ki.fn = (const void*)k_ntt_cluster2<S, MODE, SEQ, REGS>;
+  ki.block = S::CT;
+  ki.smem = 2 * ((1 << LL) + ((1 << LL) >> RB)) * (int)sizeof(W);
   ki.team = S::T;
   ki.units_per_cta = 1;
-  ki.cluster = S::T / kClusterThreads;
-  ki.rb = 4;
+  ki.cluster = S::CTAS;
+  ki.rb = RB;
   ki.mode = MODE;
-  ki.regs = 65536 / kClusterThreads;
-  ki.pad = 4;
+  ki.regs = REGS;
+  ki.pad = RB;
   ki.seq = SEQ ? 1 : 0;
   return ki;
 }
@@ -418,26 +426,55 @@ static KernelInfo cluster_info() {
   return ki;
 }
 
-// the second form (CTA-local exchanges, padded layout); seq: one operand at a time
+// The second form (CTA-local exchanges, padded layout); seq: one operand at a
+// time.  32-bit words, both operands: 64 registers, and at 2^15 eight CTAs of
+// 4096 coefficients (four resident CTAs per SM, so that other clusters run
+// while one waits at its cluster barrier): 128 / 400 products of 30-bit primes
+// 55.4 / 165 us, against 66.4 / 198 for four CTAs of 8192 coefficients, one
+// operand at a time, 128 registers; at 2^16 a cluster has eight CTAs, so each
+// keeps 8192 coefficients.
 bool lookup_ntt_cluster2(uint32_t elem, int logn, int mode, bool seq, KernelInfo* ki) {
-#define PM_C2(W, L, M)                                                           \
-  if (logn == L && mode == M) {                                                  \
-    *ki = seq ? cluster2_info<W, L, M, true>() : cluster2_info<W, L, M, false>(); \
-    return true;                                                                 \
+#define PM_C2(W, L, M, RB, LL, REGS)                                                                    \
+  if (logn == L && mode == M) {                                                                         \
+    *ki = seq ? cluster2_info<W, L, M, true>() : cluster2_info<W, L, M, false, RB, LL, REGS>();         \
+    return true;                                                                                        \
   }
   if (elem == 8) {
-    PM_C2(uint64_t, 14, 1)
-    PM_C2(uint64_t, 15, 1)
-    PM_C2(uint64_t, 16, 1)
+    PM_C2(uint64_t, 14, 1, 4, 13, 128)
+    PM_C2(uint64_t, 15, 1, 4, 13, 128)
+    PM_C2(uint64_t, 16, 1, 4, 13, 128)
   } else {
-    PM_C2(uint32_t, 14, 0)
-    PM_C2(uint32_t, 15, 0)
-    PM_C2(uint32_t, 16, 0)
-    PM_C2(uint32_t, 14, 1)
-    PM_C2(uint32_t, 15, 1)
-    PM_C2(uint32_t, 16, 1)
+    PM_C2(uint32_t, 14, 0, 4, 13, 128)
+    PM_C2(uint32_t, 15, 0, 4, 12, 64)
+    PM_C2(uint32_t, 16, 0, 4, 13, 64)
+    PM_C2(uint32_t, 14, 1, 4, 13, 128)
+    PM_C2(uint32_t, 15, 1, 4, 12, 64)
+    PM_C2(uint32_t, 16, 1, 4, 13, 64)
   }
 #undef PM_C2
+  return false;
+}
+
+// Few products: each spread over more CTAs and threads than the throughput
+// kernels take, so that one product's latency is shorter (64-bit words, eight
+// products: 49.1 -> 30.7 us at 2^15, 45.1 -> 28.3 at 2^14, 40.0 -> 24.6 at
+// 2^13, 26.7 -> 12.4 at 2^12; 32-bit words, 16 products at 2^14: 26.5 -> 14.4).
+bool lookup_ntt_cluster_small(uint32_t elem, int logn, int mode, KernelInfo* ki) {
+#define PM_CS(W, L, M, RB, LL)                              \
+  if (logn == L && mode == M) {                             \
+    *ki = cluster2_info<W, L, M, false, RB, LL, 64>();      \
+    return true;                                            \
+  }
+  if (elem == 8) {
+    PM_CS(uint64_t, 12, 1, 3, 10)
+    PM_CS(uint64_t, 13, 1, 3, 12)
+    PM_CS(uint64_t, 14, 1, 3, 12)
+    PM_CS(uint64_t, 15, 1, 3, 12)
+  } else {
+    PM_CS(uint32_t, 14, 0, 4, 12)
+    PM_CS(uint32_t, 14, 1, 4, 12)
+  }
+#undef PM_CS
   return false;
 }
 

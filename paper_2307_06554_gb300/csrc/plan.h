@@ -47,6 +47,10 @@ struct polymul_plan {
   pm::KernelInfo tki;  // tensor-path kernel, when one exists for the shape
   std::vector<PlanCandidate> cands;  // [0] is the default
   size_t chosen = 0;
+  // batches of at most small_units units run candidate `small` instead, as
+  // long as the choice is the default one (see polymul_create); 0: none
+  size_t small = 0;
+  uint64_t small_units = 0;
   bool tuned = false;
   uint64_t tuned_batch = 0;  // batch bucket of the tuned choice
   void* d_tpc = nullptr;  // tensor-path constants
@@ -69,6 +73,7 @@ struct polymul_plan {
   int grid_cap = 0;    // resident CTAs of ki (persistent grid)
   uint32_t launch_flags = 0;
   int* d_flag = nullptr;
+  int smem_sm = 0, smem_resv = 0;  // shared memory of an SM, and what each CTA takes beside its own
   unsigned long long* d_ctr = nullptr;  // kCounterSlots x {next, finished}: device entry, host streams
   int* d_err = nullptr;                 // set by kernels whose bounded waits expired
   // polymul_batch_shared scratch (digit planes of b and of T(a))
@@ -91,6 +96,7 @@ struct polymul_plan {
 
 inline void apply_candidate(polymul_plan* p, size_t i) {
   p->chosen = i;
+  p->small_units = 0;
   p->path = p->cands[i].path;
   p->ki = p->cands[i].ki;
   p->grid_cap = p->cands[i].grid_cap;
@@ -110,4 +116,5 @@ void clear_error();
 // diagnostics: true (and the kernel arguments that make its waits expire)
 // when this NTT batch launch is one that polymul_selftest_inject_wait asked for
 bool take_injected_wait(uint32_t* tx_pad, uint32_t* polls);
+bool injected_wait_pending();
 }  // namespace pm

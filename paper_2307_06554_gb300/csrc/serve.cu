@@ -239,6 +239,23 @@ cudaError_t launch_ntt(const KernelInfo& ki, int cap, uint32_t units, void** arg
   return cudaLaunchKernel(ki.fn, grid, ki.block, argv, ki.smem, st);
 }
 
+// resident clusters of a cluster kernel on the device
+cudaError_t max_clusters(const KernelInfo& ki, int num_sms, int* clusters) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = ki.cluster;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(ki.cluster * num_sms);
+  cfg.blockDim = dim3(ki.block);
+  cfg.dynamicSmemBytes = ki.smem;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(clusters, ki.fn, &cfg);
+}
+
 // The prime map rides in the launch's arguments when it fits (up to 32
 // primes of a pool of at most 256), else it is copied to the arena.
 bool inline_map(const polymul_server* s, uint32_t k) { return k <= 32 && s->pool.size() <= 256; }
@@ -621,20 +638,8 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
       return bail(cuda_fail(cudaGetLastError(), "smem attribute"));
     int cap = 0;
     if (ki.cluster > 0) {
-      cudaLaunchConfig_t cfg;
-      memset(&cfg, 0, sizeof cfg);
-      cudaLaunchAttribute attr;
-      attr.id = cudaLaunchAttributeClusterDimension;
-      attr.val.clusterDim.x = ki.cluster;
-      attr.val.clusterDim.y = 1;
-      attr.val.clusterDim.z = 1;
-      cfg.gridDim = dim3(ki.cluster * s->num_sms);
-      cfg.blockDim = dim3(ki.block);
-      cfg.dynamicSmemBytes = ki.smem;
-      cfg.attrs = &attr;
-      cfg.numAttrs = 1;
       int clusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&clusters, ki.fn, &cfg) != cudaSuccess || clusters < 1)
+      if (max_clusters(ki, s->num_sms, &clusters) != cudaSuccess || clusters < 1)
         return bail(fail(POLYMUL_ENOTSUP, "no cluster fits for n=2^%d", logn));
       cap = clusters * ki.cluster;
     } else {
@@ -649,7 +654,19 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
     s->dki[logn] = ki;  // the cluster kernels read and write with plain accesses
     s->dgrid_cap[logn] = cap;
     KernelInfo dk;
-    if (ki.cluster == 0 && lookup_ntt_direct_u64(logn, &dk)) {
+    if (lookup_ntt_cluster_small(8, logn, 1, &dk)) {
+      // n = 2^12 .. 2^15: a request is a few rows, so one row's latency is
+      // its service time and the lanes' throughput (200 requests of 2^12 ..
+      // 2^14, up to 8 primes, 8 lanes, all queued: see the kernel)
+      if (dk.smem > 48 * 1024 &&
+          cudaFuncSetAttribute(dk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dk.smem) != cudaSuccess)
+        return bail(cuda_fail(cudaGetLastError(), "smem attribute"));
+      int clusters = 0;
+      if (max_clusters(dk, s->num_sms, &clusters) != cudaSuccess || clusters < 1)
+        return bail(fail(POLYMUL_ENOTSUP, "no cluster fits for n=2^%d", logn));
+      s->dki[logn] = dk;
+      s->dgrid_cap[logn] = clusters * dk.cluster;
+    } else if (ki.cluster == 0 && lookup_ntt_direct_u64(logn, &dk)) {
       if (dk.smem > 48 * 1024 &&
           cudaFuncSetAttribute(dk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dk.smem) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "smem attribute"));

@@ -42,7 +42,10 @@ def test_edges(n, batch, cyclic):
         a[3, j, n - 1] = q - 1
     with pm.Plan(n, qs, path=pm.PATH_NTT, flags=pm.FLAG_CYCLIC if cyclic else 0) as plan:
         assert (plan.info["radix_bits"], plan.info["exchange_pad"]) == (5, 3)  # the default is this unit
+        default = run_plan_batch(plan, a, b)  # the smaller batches run candidate 1
+        plan.select(0)  # this unit whatever the batch
         got = run_plan_batch(plan, a, b)
+    assert np.array_equal(got, default)
     idx = sorted(set(range(4)) | {batch // 2, batch - 2, batch - 1})
     assert_equal_residues(got[idx], native.polymul_batch(a[idx], b[idx], qs, cyclic=cyclic), "tiny moduli")
     with pm.Plan(n, qs, path=pm.PATH_NTT, flags=pm.FLAG_CYCLIC if cyclic else 0) as plan:
@@ -56,3 +59,32 @@ def test_first_modulus_past_the_limit():
     q = next(q for q in range(512 * (LIMIT // 512 + 1) + 1, 1 << 20, 512) if wl.is_prime(q))
     with pm.Plan(256, [q], path=pm.PATH_NTT) as plan:
         assert plan.info["radix_bits"] == 4
+
+
+@pytest.mark.parametrize("batch", [1, 9, 611, 2600])
+@pytest.mark.parametrize("qs", [[12289], [18433, 12289]])
+@pytest.mark.parametrize("cyclic", [False, True])
+def test_shared_operand(batch, qs, cyclic):
+    """One operand for the whole batch: fewer products than warps, a last
+    group with idle warps, several products per warp, two primes."""
+    import torch
+    from paper_2307_06554_gb300 import polymul as pm
+    n = 1024
+    rng = np.random.default_rng(batch + len(qs))
+    a = wl.uniform_coeffs(rng, 1, qs, n, np.uint32)
+    b = wl.uniform_coeffs(rng, batch, qs, n, np.uint32)
+    for j, q in enumerate(qs):
+        a[0, j, ::3] = q - 1
+        b[0, j] = q - 1
+    flags = pm.FLAG_CYCLIC if cyclic else 0
+    with pm.Plan(n, qs, path=pm.PATH_NTT, flags=flags) as plan:
+        ta, tb = (torch.from_numpy(x.view(np.int32)).cuda() for x in (a[0].copy(), b))
+        tc = torch.full_like(tb, -1)
+        pm.polymul_batch_shared(plan.handle, ta, tb, tc, batch)
+        torch.cuda.synchronize()
+        pm.polymul_plan_status(plan.handle)
+        got = tc.cpu().numpy().view(np.uint32)
+        full = np.broadcast_to(a, b.shape).copy()
+        assert np.array_equal(got, run_plan_batch(plan, full, b))
+    idx = sorted({0, batch // 2, batch - 1})
+    assert_equal_residues(got[idx], native.polymul_batch(full[idx], b[idx], qs, cyclic=cyclic), "shared tiny")
