@@ -50,7 +50,7 @@ inline void build_ntt_tables_into(uint64_t q, uint32_t n, W* twf, W* twi, PrimeC
   pc.scale_p = (W)shoup_companion(scale, q, bits);
   pc.scale_w = (W)scale_w;
   pc.scale_wp = (W)shoup_companion(scale_w, q, bits);
-  pc.zero = 0;
+  pc.pad = 0;
 }
 
 template <typename W>

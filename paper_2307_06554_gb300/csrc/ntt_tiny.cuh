@@ -231,33 +231,29 @@ __device__ __forceinline__ void tiny_ring(int* b, const int (&a)[8], int wz, con
   });
 }
 
-// One unit: c = a b mod (x^n +- 1, q).  Interface as polymul_unit; twf and
-// twi are tables of n / 8 words (see build_tiny_tables), pc.scale_p the word
-// of 1, pc.scale and pc.scale_w those of the last inverse stage.
+// One operand through the forward transform and back to centred residues (the
+// low layout).
+template <class S, class Sync>
+__device__ __forceinline__ void tiny_transform(int (&x)[32], const uint32_t* in, int* s, const int* __restrict__ tw,
+                                               const PrimeConst<uint32_t>& pc, uint32_t t, Sync sync) {
+  const TinyMod m{(int)pc.q, (int)pc.qinv};
+  tiny_forward<S>(x, in, s, tw, m, t, sync);
+  sfor<0, 32>([&](auto ec) {
+    constexpr int e = decltype(ec)::value;
+    x[e] = tiny_mul(x[e], (int)pc.scale_p, m);
+  });
+}
+
+// From b's transform in x and a's at sa (low layout): products, inverse
+// through the exchange buffer sb, results to c.  `hook` as for polymul_unit.
 template <class S, class Sync, class Hook>
-__device__ __forceinline__ void polymul_unit_tiny(uint32_t* __restrict__ c, const int* __restrict__ twf,
-                                                  const int* __restrict__ twi, const PrimeConst<uint32_t>& pc,
-                                                  uint32_t* sa_, uint32_t* sb_, const uint32_t* ia, const uint32_t* ib,
-                                                  uint32_t t, bool act, Sync sync, Hook&& hook) {
+__device__ __forceinline__ void tiny_finish(uint32_t* __restrict__ c, int (&x)[32], const int* sa, int* sb,
+                                            const int* __restrict__ twf, const int* __restrict__ twi,
+                                            const PrimeConst<uint32_t>& pc, uint32_t t, bool act, Sync sync,
+                                            Hook&& hook) {
   using TS = TinyShape<S>;
-  int* sa = reinterpret_cast<int*>(sa_);
-  int* sb = reinterpret_cast<int*>(sb_);
   const TinyMod m{(int)pc.q, (int)pc.qinv};
   const int one = (int)pc.scale_p;
-  int x[32];
-  // a, then b, through the same instructions (a body of its own for each
-  // would be fetched twice: the warps of an SM run through it at different
-  // places, and instruction fetch was the first of its stalls)
-#pragma unroll 1
-  for (int op = 0; op < 2; ++op) {
-    int* s = op ? sb : sa;
-    tiny_forward<S>(x, op ? ib : ia, s, twf, m, t, sync);
-    sfor<0, 32>([&](auto ec) {
-      constexpr int e = decltype(ec)::value;
-      x[e] = tiny_mul(x[e], one, m);
-    });
-    if (op == 0) tiny_st16(s + 36 * t, x);  // a parked where this thread alone loaded it
-  }
   // products: rings 2 i and 2 i + 1 of this thread are x^8 - z and x^8 + z
   // for the root z of the stage above
   int wz[2];
@@ -341,6 +337,29 @@ __device__ __forceinline__ void polymul_unit_tiny(uint32_t* __restrict__ c, cons
       c[t + TS::T * e] = __viaddmin_u32((uint32_t)x[e], pc.q, (uint32_t)x[e]);
     });
   }
+}
+
+// One unit: c = a b mod (x^n +- 1, q).  Interface as polymul_unit; twf and
+// twi are tables of n / 8 words (see build_tiny_tables), pc.scale_p the word
+// of 1, pc.scale and pc.scale_w those of the last inverse stage.
+template <class S, class Sync, class Hook>
+__device__ __forceinline__ void polymul_unit_tiny(uint32_t* __restrict__ c, const int* __restrict__ twf,
+                                                  const int* __restrict__ twi, const PrimeConst<uint32_t>& pc,
+                                                  uint32_t* sa_, uint32_t* sb_, const uint32_t* ia, const uint32_t* ib,
+                                                  uint32_t t, bool act, Sync sync, Hook&& hook) {
+  int* sa = reinterpret_cast<int*>(sa_);
+  int* sb = reinterpret_cast<int*>(sb_);
+  int x[32];
+  // a, then b, through the same instructions (a body of its own for each
+  // would be fetched twice: the warps of an SM run through it at different
+  // places, and instruction fetch was the first of its stalls)
+#pragma unroll 1
+  for (int op = 0; op < 2; ++op) {
+    int* s = op ? sb : sa;
+    tiny_transform<S>(x, op ? ib : ia, s, twf, pc, t, sync);
+    if (op == 0) tiny_st16(s + 36 * t, x);  // a parked where this thread alone loaded it
+  }
+  tiny_finish<S>(c, x, sa, sb, twf, twi, pc, t, act, sync, hook);
 }
 
 }  // namespace pm

@@ -14,7 +14,7 @@ struct alignas(16) PrimeConst {
   W scale_p;   // Shoup companion of scale
   W scale_w;   // psi^-brv(1) * scale mod q (last inverse stage twiddle)
   W scale_wp;  // Shoup companion of scale_w
-  W zero;      // 0, as a value the compiler cannot know (see polymul_unit_seq)
+  W pad;
 };
 
 // One (product, prime) row of an uneven list: its element offset in a, b, c
@@ -122,6 +122,21 @@ struct NttSharedArgs {
   uint32_t k;
   uint32_t tw_stride;
   unsigned long long* ctr;  // {next, finished}, zero between launches
+  int* err;
+};
+
+// Shared-operand products of the smallest moduli (k_ntt_tiny_shared).
+struct TinySharedArgs {
+  const uint32_t* a;  // [k][n]
+  const uint32_t* b;  // [batch][k][n]
+  uint32_t* c;
+  const int* tw_fwd;  // [k][n / 8] words (build_tiny_tables)
+  const int* tw_inv;
+  const PrimeConst<uint32_t>* pc;
+  uint64_t batch;
+  uint32_t k;
+  uint32_t ctas_per_prime;  // work item v: prime v / ctas_per_prime, every
+                            // ctas_per_prime-th group of eight products
   int* err;
 };
 

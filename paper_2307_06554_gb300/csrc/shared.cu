@@ -372,6 +372,24 @@ static int shared_ntt(polymul_plan* p, const void* a, const void* b, void* c, ui
   KernelInfo prep, kmain;
   if (p->elem != 4 || p->aux_prime || p->ki.cluster || !lookup_ntt_shared((int)p->logn, p->mode, &prep, &kmain))
     return fail(POLYMUL_ENOTSUP, "shared-operand NTT products need 32-bit words, n in [1024, 8192] and a direct NTT");
+  if (p->d_tiny_f && lookup_ntt_tiny_shared((int)p->logn, &kmain)) {
+    int per_sm = 0;
+    if (kmain.smem > 48 * 1024)
+      PM_CUDA(cudaFuncSetAttribute(kmain.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kmain.smem));
+    PM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kmain.fn, kmain.block, kmain.smem));
+    if (per_sm < 1) return fail(POLYMUL_ENOTSUP, "shared-operand NTT kernel does not fit on an SM");
+    const uint64_t cap = (uint64_t)per_sm * p->num_sms;
+    const uint64_t groups = (batch + kmain.units_per_cta - 1) / kmain.units_per_cta;
+    const uint64_t cpp = std::max<uint64_t>(1, std::min<uint64_t>(groups, cap / p->k));
+    TinySharedArgs ta{(const uint32_t*)a, (const uint32_t*)b, (uint32_t*)c, (const int*)p->d_tiny_f,
+                      (const int*)p->d_tiny_i, (const PrimeConst<uint32_t>*)p->d_tiny_pc, batch, p->k, (uint32_t)cpp,
+                      p->d_err};
+    void* argv_t[] = {&ta};
+    // the next batch launch on the stream waits for this one in full
+    StreamOrderGuard order(p->device, st);
+    order.record(nullptr);
+    return pdl_launch(kmain.fn, (int)std::min<uint64_t>(cpp * p->k, cap), kmain.block, kmain.smem, argv_t, st);
+  }
   const size_t ahat_bytes = (size_t)p->k * p->n * 4;
   int rc = sh_scratch(p, 256 + ahat_bytes);
   if (rc != POLYMUL_OK) return rc;
