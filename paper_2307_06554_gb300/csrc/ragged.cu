@@ -39,15 +39,17 @@ struct TeamSync {
 // per list by measurement (polymul_ragged_tune):
 //   set 0: the XOR-swizzled exchange layout, both operands in registers;
 //   set 1: the padded layout (one word after every 2^RB, a base register
-//          plus constant offsets per layout), one operand in registers at a
-//          time for 2^10, 2^11 (as the homogeneous kernels measured) and for
-//          2^14, whose 32 coefficients per operand and thread otherwise spill.
+//          plus constant offsets per layout); 2^10 .. 2^13 at 64 registers,
+//          two CTAs and 32 warps per SM (the multiply pipe is the bound, and
+//          16 warps left it idle at barriers and exchanges: the 2000-product
+//          list 1.045 -> 0.895 ms with this set and the batch kernel for
+//          2^14); 2^14 one operand in registers at a time.
 constexpr int ragged_rb(int logn) { return logn <= 13 ? 4 : 5; }
 template <int LOGN, int SET>
 using RaggedShape = Shape<uint32_t, LOGN, ragged_rb(LOGN), SET == 1 ? ragged_rb(LOGN) : 0>;
 template <int LOGN, int SET>
 constexpr bool ragged_seq() {
-  return SET == 1 && (LOGN == 10 || LOGN == 11 || LOGN == 14);
+  return SET == 1 && LOGN == 14;
 }
 
 // One degree segment: the units of degree 2^LOGN, taken one at a time by
@@ -121,7 +123,7 @@ __device__ __forceinline__ bool ragged_segment(const RaggedArgs& args, const Rag
 // coefficients per thread) has a kernel of its own, so that its register
 // pressure (and the spills it causes) does not reach the other degrees.
 template <int MODE, int LO, int HI, int SET>
-__global__ void __launch_bounds__(kRaggedThreads, 1) k_ntt_ragged(RaggedArgs args) {
+__global__ void __launch_bounds__(kRaggedThreads, (SET == 1 && HI <= 13) ? 2 : 1) k_ntt_ragged(RaggedArgs args) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t mbar[kRaggedMaxTeams];
   __shared__ unsigned long long s_next[kRaggedMaxTeams];

@@ -69,9 +69,9 @@ struct polymul_ragged_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraphNode_t node[2] = {nullptr, nullptr};
-  // shape set of each launch: the padded one-operand set by default (fewer
-  // registers, no spills at 2^14); polymul_ragged_tune measures both
-  int set[2] = {1, 1};
+  // shape set of each launch: the padded set for 2^10 .. 2^13, the batch
+  // kernel for 2^14 by default; polymul_ragged_tune measures both
+  int set[2] = {1, 0};
   // degree segments of the whole list (host copy; d_items holds those the
   // NTT launches take), and the classes on the tensor path (bit logn - 10)
   std::vector<RaggedItem> items_h;
@@ -212,8 +212,8 @@ extern "C" int polymul_ragged_create(const uint64_t* pool, uint32_t pool_size, u
   for (int set = 0; set < kRaggedSets && rc == POLYMUL_OK; ++set)
     if (!lookup_ntt_ragged(r->mode, set, &r->ki[set][0], &r->ki[set][1])) rc = fail(POLYMUL_ENOTSUP, "no ragged kernel");
   // the 2^14 segment's set 0: the homogeneous one-CTA-per-product kernel
-  // with a row table (measured 504 vs 555 us for the 2000-product list's
-  // 2^14 rows; it spills less at the 128 registers a 512-thread CTA allows)
+  // with a row table (it spills nothing at the 128 registers a 512-thread CTA
+  // allows; the one-operand kernel of set 1 316 bytes a thread)
   if (rc == POLYMUL_OK && r->lognmax >= 14 && lookup_ntt_u32_rb5(14, r->mode, &r->ki[0][1])) r->batch14 = true;
   if (rc == POLYMUL_OK) {
     cudaError_t e = cudaGetDevice(&r->device);
