@@ -62,8 +62,10 @@ namespace {
 
 // Tables for the NTT primes: the plan's moduli, or (auxiliary-prime mode)
 // the single auxiliary prime.
+// `tiny` (32-bit words): behind them, in the same allocations, the tables of
+// the unit for the smallest moduli (ntt_tiny.cuh).
 template <typename W>
-int upload_ntt_tables(polymul_plan* p) {
+int upload_ntt_tables(polymul_plan* p, bool tiny = false) {
   const std::vector<uint64_t> primes = p->aux_prime ? std::vector<uint64_t>{p->aux_prime} : p->q;
   const uint32_t np = (uint32_t)primes.size();
   std::vector<W> all_f, all_i, f, i;
@@ -75,6 +77,17 @@ int upload_ntt_tables(polymul_plan* p) {
     all_f.insert(all_f.end(), f.begin(), f.end());
     all_i.insert(all_i.end(), i.begin(), i.end());
   }
+  const size_t words = all_f.size();  // 2 n np: the tables behind them start 16-byte aligned
+  if constexpr (sizeof(W) == 4) {
+    if (tiny) {
+      pcs.resize(2 * np);
+      for (uint32_t j = 0; j < np; ++j) {
+        build_tiny_tables(primes[j], p->n, f, i, pcs[np + j], p->cyclic);
+        all_f.insert(all_f.end(), f.begin(), f.end());
+        all_i.insert(all_i.end(), i.begin(), i.end());
+      }
+    }
+  }
   const size_t tb = all_f.size() * sizeof(W);
   PM_CUDA(cudaMalloc(&p->d_twf, tb));
   PM_CUDA(cudaMalloc(&p->d_twi, tb));
@@ -82,32 +95,17 @@ int upload_ntt_tables(polymul_plan* p) {
   PM_CUDA(cudaMemcpy(p->d_twf, all_f.data(), tb, cudaMemcpyHostToDevice));
   PM_CUDA(cudaMemcpy(p->d_twi, all_i.data(), tb, cudaMemcpyHostToDevice));
   PM_CUDA(cudaMemcpy(p->d_pc, pcs.data(), pcs.size() * sizeof(PrimeConst<W>), cudaMemcpyHostToDevice));
+  if (tiny) {
+    p->d_tiny_f = static_cast<W*>(p->d_twf) + words;
+    p->d_tiny_i = static_cast<W*>(p->d_twi) + words;
+    p->d_tiny_pc = static_cast<PrimeConst<W>*>(p->d_pc) + np;
+  }
   if (p->aux_prime) {
     std::vector<W> qs(p->q.begin(), p->q.end());
     PM_CUDA(cudaMalloc(&p->d_outer, qs.size() * sizeof(W)));
     PM_CUDA(cudaMemcpy(p->d_outer, qs.data(), qs.size() * sizeof(W), cudaMemcpyHostToDevice));
   }
   return POLYMUL_OK;
-}
-
-// Tables of the unit for the smallest moduli (ntt_tiny.cuh).
-int upload_tiny_tables(polymul_plan* p) {
-  std::vector<uint32_t> all_f, all_i, f, i;
-  std::vector<PrimeConst<uint32_t>> pcs(p->k);
-  for (uint32_t j = 0; j < p->k; ++j) {
-    build_tiny_tables(p->q[j], p->n, f, i, pcs[j], p->cyclic);
-    all_f.insert(all_f.end(), f.begin(), f.end());
-    all_i.insert(all_i.end(), i.begin(), i.end());
-  }
-  auto up = [](void** dst, const void* src, size_t bytes) -> int {
-    PM_CUDA(cudaMalloc(dst, bytes));
-    PM_CUDA(cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice));
-    return POLYMUL_OK;
-  };
-  int r = up(&p->d_tiny_f, all_f.data(), all_f.size() * sizeof(uint32_t));
-  if (r == POLYMUL_OK) r = up(&p->d_tiny_i, all_i.data(), all_i.size() * sizeof(uint32_t));
-  if (r == POLYMUL_OK) r = up(&p->d_tiny_pc, pcs.data(), pcs.size() * sizeof(pcs[0]));
-  return r;
 }
 
 // Auxiliary NTT prime for moduli without a 2n-th root of unity: the largest
@@ -510,15 +508,13 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
               n, p->cyclic ? "n" : "2n");
   } else {
     // the default kernel first, then the candidates the autotuner may prefer
-    rc = p->elem == 4 ? upload_ntt_tables<uint32_t>(p) : upload_ntt_tables<uint64_t>(p);
     KernelInfo v;
-    const KernelInfo word = p->ki;
     // moduli below 18500 (12289 and the like), n = 2^8 .. 2^10: the unit of
     // ntt_tiny.cuh first (see there for the bound and the measurements)
-    if (rc == POLYMUL_OK && p->elem == 4 && qmax < kTinyQMax && lookup_ntt_tiny((int)p->logn, &v)) {
-      rc = upload_tiny_tables(p);
-      if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, v);
-    }
+    const bool tiny = p->elem == 4 && qmax < kTinyQMax && lookup_ntt_tiny((int)p->logn, &v);
+    rc = p->elem == 4 ? upload_ntt_tables<uint32_t>(p, tiny) : upload_ntt_tables<uint64_t>(p);
+    const KernelInfo word = p->ki;
+    if (rc == POLYMUL_OK && tiny) rc = add_candidate(POLYMUL_PATH_NTT, v);
     if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, word);
     if (rc == POLYMUL_OK && p->elem == 4 && lookup_ntt_u32_rb5((int)p->logn, p->mode, &v) && v.fn != p->cands[0].ki.fn)
       rc = add_candidate(POLYMUL_PATH_NTT, v);
@@ -620,9 +616,6 @@ extern "C" void polymul_destroy(polymul_plan* p) {
   cudaFree(p->d_twf);
   cudaFree(p->d_twi);
   cudaFree(p->d_pc);
-  cudaFree(p->d_tiny_f);
-  cudaFree(p->d_tiny_i);
-  cudaFree(p->d_tiny_pc);
   cudaFree(p->d_tpc);
   cudaFree(p->d_tpc8);
   cudaFree(p->d_tp64);

@@ -40,6 +40,7 @@ struct polymul_plan {
   void* d_twi = nullptr;
   void* d_pc = nullptr;
   // the same for the unit of the smallest moduli, when a candidate uses it
+  // (parts of the three allocations above)
   void* d_tiny_f = nullptr;
   void* d_tiny_i = nullptr;
   void* d_tiny_pc = nullptr;
