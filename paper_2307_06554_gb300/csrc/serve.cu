@@ -113,8 +113,19 @@ struct polymul_server {
   // streams of their own joined by events, so that a request's copies in do
   // not wait for the previous request's kernel and copy out on the lane
   std::vector<cudaStream_t> lanes, lanes_in, lanes_out;
-  unsigned long long* d_ctr = nullptr;  // 2 per lane
-  int* d_err = nullptr;                 // one error word per lane
+  // A direct request is one kernel, so it needs one stream, not a pipeline:
+  // it may take any of a lane's three.  Queue q: 0 .. nlanes - 1 the kernel
+  // streams (a staged request's lane is the queue of its kernel), then the
+  // copy-in, then the copy-out streams.  A request's kernel spends most of
+  // its time waiting for the host link, so three times as many of them in
+  // flight keep the link busier (200 requests of 2^12 .. 2^14, up to 8
+  // primes, 8 lanes: 1.23 ms on the kernel streams alone, 1.10 with the others).
+  int direct_queues() const { return 3 * nlanes; }
+  cudaStream_t queue_stream(int q) const {
+    return q < nlanes ? lanes[q] : q < 2 * nlanes ? lanes_in[q - nlanes] : lanes_out[q - 2 * nlanes];
+  }
+  unsigned long long* d_ctr = nullptr;  // 2 per queue
+  int* d_err = nullptr;                 // one error word per queue
   int* h_err = nullptr;                 // page-locked, one per in-flight slot
   // where the device supports native atomics on host memory, h_err is also
   // mapped into the device's address space (d_err_mapped): each request's
@@ -264,7 +275,7 @@ bool inline_map(const polymul_server* s, uint32_t k) { return k <= 32 && s->pool
 // writes c in host memory; then its error word and the completion event
 // (server thread)
 cudaError_t issue_direct(polymul_server* s, ServeReq* r) {
-  cudaStream_t st = s->lanes[r->lane];
+  cudaStream_t st = s->queue_stream(r->lane);
   cudaError_t e;
   uint32_t* dmap = nullptr;
   if (!inline_map(s, r->k)) {
@@ -380,6 +391,7 @@ void server_loop(polymul_server* s) {
   cudaSetDevice(s->device);
   std::vector<ServeReq*> done;
   std::string err_msg;
+  int scan = 0;  // the queue whose oldest request is looked at next
   while (!s->stop.load()) {
     bool progress = false;
     const double t_pass = now_s();
@@ -392,9 +404,13 @@ void server_loop(polymul_server* s) {
         s->queue.pop_front();
       }
     }
-    // retire: only the oldest request of each lane can be the next to finish
-    for (int l = 0; l < s->nlanes; ++l) {
-      std::deque<ServeReq*>& f = s->lane_fifo[l];
+    // retire: only the oldest request of each queue can be the next to
+    // finish; at most as many queues per pass as there are lanes, in turn, so
+    // that the event queries of a pass between two admissions stay few
+    for (int i = 0, looked = 0; i < s->direct_queues() && looked < s->nlanes; ++i) {
+      std::deque<ServeReq*>& f = s->lane_fifo[scan];
+      scan = scan + 1 == s->direct_queues() ? 0 : scan + 1;
+      if (!f.empty()) ++looked;
       while (!f.empty()) {
         ServeReq* r = f.front();
         const cudaError_t q = cudaEventQuery(r->ev);
@@ -429,6 +445,13 @@ void server_loop(polymul_server* s) {
       int lane = 0;
       for (int l = 1; l < s->nlanes; ++l)
         if (s->lane_bytes[l] < s->lane_bytes[lane]) lane = l;
+      // A direct request that moves half a MB or more finds another queue
+      // when every lane is busy.  Smaller ones keep to the lanes: there the
+      // server thread's issue time is the bound, and launches on more streams
+      // cost it more (1000 requests of 2^10 .. 2^12: 4.4 -> 4.7 us each).
+      if (r->direct && r->weight >= (512u << 10) && s->lane_bytes[lane] > 0)
+        for (int l = s->nlanes; l < s->direct_queues(); ++l)
+          if (s->lane_bytes[l] < s->lane_bytes[lane]) lane = l;
       r->lane = lane;
       s->lane_bytes[lane] += r->weight;
       take_events(s, r);
@@ -584,8 +607,9 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
   s->lognmax = __builtin_ctz(n_max);
   s->pool.assign(pool, pool + pool_size);
   s->nlanes = (int)lanes;
-  s->lane_bytes.assign(lanes, 0);
-  s->lane_fifo.resize(lanes);
+  const size_t queues = (size_t)s->direct_queues();
+  s->lane_bytes.assign(queues, 0);
+  s->lane_fifo.resize(queues);
   s->max_inflight = std::max<size_t>(64, 8 * (size_t)lanes);  // enough requests to keep every lane busy
   int rc = POLYMUL_OK;
   auto bail = [&](int code) {
@@ -603,8 +627,8 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
     return bail(cuda_fail(cudaGetLastError(), "device query"));
   if (cudaMalloc(&s->d_twf, twf.size() * 8) != cudaSuccess || cudaMalloc(&s->d_twi, twi.size() * 8) != cudaSuccess ||
       cudaMalloc(&s->d_pc, pcs.size() * sizeof(PrimeConst<uint64_t>)) != cudaSuccess ||
-      cudaMalloc(&s->d_ctr, 2 * lanes * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMalloc(&s->d_err, lanes * sizeof(int)) != cudaSuccess ||
+      cudaMalloc(&s->d_ctr, 2 * queues * sizeof(unsigned long long)) != cudaSuccess ||
+      cudaMalloc(&s->d_err, queues * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&s->d_arena, device_bytes) != cudaSuccess ||
       cudaHostAlloc(&s->h_err, s->max_inflight * sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
       cudaHostAlloc(&s->h_map, s->max_inflight * pool_size * sizeof(uint32_t), cudaHostAllocDefault) != cudaSuccess)
@@ -623,8 +647,8 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
       cudaMemcpy(s->d_twi, twi.data(), twi.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(s->d_pc, pcs.data(), pcs.size() * sizeof(PrimeConst<uint64_t>), cudaMemcpyHostToDevice) !=
           cudaSuccess ||
-      cudaMemset(s->d_ctr, 0, 2 * lanes * sizeof(unsigned long long)) != cudaSuccess ||
-      cudaMemset(s->d_err, 0, lanes * sizeof(int)) != cudaSuccess)
+      cudaMemset(s->d_ctr, 0, 2 * queues * sizeof(unsigned long long)) != cudaSuccess ||
+      cudaMemset(s->d_err, 0, queues * sizeof(int)) != cudaSuccess)
     return bail(cuda_fail(cudaGetLastError(), "table upload"));
   s->arena_bytes = device_bytes;
   s->free_list[0] = device_bytes;
@@ -657,7 +681,8 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
     if (lookup_ntt_cluster_small(8, logn, 1, &dk)) {
       // n = 2^12 .. 2^15: a request is a few rows, so one row's latency is
       // its service time and the lanes' throughput (200 requests of 2^12 ..
-      // 2^14, up to 8 primes, 8 lanes, all queued: see the kernel)
+      // 2^14, up to 8 primes, 8 lanes, all queued: 1.49 ms with the batch
+      // kernel's direct form and the throughput cluster kernels, 1.23 so)
       if (dk.smem > 48 * 1024 &&
           cudaFuncSetAttribute(dk.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dk.smem) != cudaSuccess)
         return bail(cuda_fail(cudaGetLastError(), "smem attribute"));
