@@ -137,7 +137,8 @@ typedef struct polymul_plan_info {
                              is in effect for it                            */
     uint32_t ntt_mode;    /* NTT path: reduction mode of the main kernel:
                              0 = values in [0, 2q), 1 = [0, 4q) (Harvey),
-                             2 = unreduced (small q)                        */
+                             2 = unreduced (small q), 4 = 64-bit words
+                             below 2^59, values in [0, 32q)                 */
     uint32_t regs;        /* NTT path: register budget per thread of the main
                              kernel (fewer registers, more resident warps)  */
     uint32_t cyclic;      /* 1: the ring Z_q[x]/(x^n-1); 0: Z_q[x]/(x^n+1) */

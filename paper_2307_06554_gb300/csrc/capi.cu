@@ -305,6 +305,10 @@ int upload_tensor_tables(polymul_plan* p) {
   return r;
 }
 
+// The second cluster form has no unreduced mode; the next one's bounds hold
+// for its moduli too.
+int cluster_mode(uint32_t elem, int mode) { return mode != 2 ? mode : elem == 8 ? 4 : 1; }
+
 bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
   // n = 2^14, 32-bit words: one 512-thread CTA per product (32 coefficients
   // per thread) beats the two-CTA cluster (measured 101.9 vs 160.8 us for
@@ -314,9 +318,8 @@ bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
     // beyond one CTA: one product per thread-block cluster, the form with
     // CTA-local exchanges (measured on GB300 against the first form: 64-bit
     // words with both operands in registers 1.38-1.49x faster at 2^14 ..
-    // 2^16; 32-bit words see lookup_ntt_cluster2); the unreduced mode takes
-    // the Harvey-bound kernels, whose bounds hold for its moduli too
-    if (lookup_ntt_cluster2(elem, logn, mode == 2 ? 1 : mode, false, ki)) return true;
+    // 2^16; 32-bit words see lookup_ntt_cluster2)
+    if (lookup_ntt_cluster2(elem, logn, cluster_mode(elem, mode), false, ki)) return true;
     return lookup_ntt_cluster(elem, logn, mode, ki) || (mode == 2 && lookup_ntt_cluster(elem, logn, 1, ki));
   }
   if (elem == 4) {
@@ -325,6 +328,7 @@ bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
     return lookup_ntt_u32_m2(logn, ki);
   }
   if (mode == 1) return lookup_ntt_u64_m1(logn, ki);
+  if (mode == 4) return lookup_ntt_u64_m4(logn, ki);
   if (mode == 2) return lookup_ntt_u64_m2(logn, ki);
   return false;
 }
@@ -524,7 +528,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     // the cluster kernels not already the default: the second form's other
     // operand scheme, and the first form
     if (p->logn >= 14) {
-      const int cm = p->mode == 2 ? 1 : p->mode;
+      const int cm = cluster_mode(p->elem, p->mode);
       for (int seq = 0; seq < 2; ++seq)
         if (rc == POLYMUL_OK && lookup_ntt_cluster2(p->elem, (int)p->logn, cm, seq != 0, &v) &&
             v.fn != p->cands[0].ki.fn)
@@ -554,7 +558,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     // 26.6 / 40.6, 111 products 43.1 / 41.0.  32-bit words at 2^14: 64
     // products 18.7 / 25.3, 111 products 28.2 / 25.7.
     if (rc == POLYMUL_OK && p->logn >= (p->elem == 8 ? 13u : 14u) &&
-        lookup_ntt_cluster_small(p->elem, (int)p->logn, p->mode == 2 ? 1 : p->mode, &v)) {
+        lookup_ntt_cluster_small(p->elem, (int)p->logn, cluster_mode(p->elem, p->mode), &v)) {
       rc = add_candidate(POLYMUL_PATH_NTT, v);
       few = p->cands.size() - 1;
     }

@@ -14,7 +14,7 @@ struct KernelInfo {
   int tmem_cols = 0;         // tensor-memory columns allocated per CTA (0: none)
   int cluster = 0;           // CTAs per thread-block cluster (0: no cluster launch)
   int rb = 0;                // NTT: stage bits per register pass
-  int mode = 0;              // NTT: reduction mode (0..2, see ntt.cuh)
+  int mode = 0;              // NTT: reduction mode (0..2, 4, see ntt.cuh)
   int regs = 0;              // NTT: register budget per thread
   int pad = 0;               // NTT: exchange layout (0 XOR swizzle, s > 0 one padding word per 2^s)
   int seq = 0;               // NTT: 1 = one operand in registers at a time
@@ -28,12 +28,13 @@ struct KernelInfo {
 };
 
 // batched negacyclic NTT, k_ntt_batch<W, LOGN, MODE> (MODE: 0 = kQ31,
-// 1 = kL4, 2 = kSmall; see ntt.cuh)
+// 1 = kL4, 2 = kSmall, 4 = kLazy; see ntt.cuh)
 bool lookup_ntt_u32_m0(int logn, KernelInfo* ki);  // logn 4..14
 bool lookup_ntt_u32_m1(int logn, KernelInfo* ki);
 bool lookup_ntt_u32_m2(int logn, KernelInfo* ki);
 bool lookup_ntt_u64_m1(int logn, KernelInfo* ki);  // logn 4..13
 bool lookup_ntt_u64_m2(int logn, KernelInfo* ki);
+bool lookup_ntt_u64_m4(int logn, KernelInfo* ki);
 bool lookup_ntt_tiny(int logn, KernelInfo* ki);     // moduli below 18500, logn 8..10
 bool lookup_ntt_u32_aux(int logn, KernelInfo* ki);  // auxiliary-prime mode, logn 4..14
 bool lookup_ntt_u32_aux_rb2(int logn, KernelInfo* ki);  // the same with radix-4 passes, logn 7..10

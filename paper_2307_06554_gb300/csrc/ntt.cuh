@@ -136,12 +136,19 @@ __device__ __forceinline__ uint32_t xpos(uint32_t j) {
 //          double per stage (2^(s+1) q after s stages), the subtraction
 //          offset of stage s being that bound;
 //   kTiny  q < 18500, n = 2^8 .. 2^10: the unit of ntt_tiny.cuh (signed
-//          residues, its own tables).
-enum { kQ31 = 0, kL4 = 1, kSmall = 2, kTiny = 3 };
+//          residues, its own tables);
+//   kLazy  64-bit words, q < 2^59: a word holds 32q, so the forward values
+//          grow by 2q per stage to at most 31q in 15 stages with no
+//          conditional subtraction (six instructions on a 64-bit value); the
+//          inverse doubles a value per stage without a multiplication inside
+//          a pass of at most four stages, from 2q to at most 32q, and brings
+//          it back below 2q at the pass's end (15 subtractions per 16
+//          coefficients and four stages instead of 32).
+enum { kQ31 = 0, kL4 = 1, kSmall = 2, kTiny = 3, kLazy = 4 };
 
 template <typename W, int MODE>
 __device__ __forceinline__ void ct_bfly(W& x, W& y, const TwPair<W>& w, const PrimeConst<W>& pc) {
-  if constexpr (MODE == kSmall) {
+  if constexpr (MODE == kSmall || MODE == kLazy) {
     W t = shoup(y, w.w, w.wp, pc.q);
     y = x - t + pc.q2;
     x = x + t;
@@ -158,10 +165,30 @@ __device__ __forceinline__ void ct_bfly(W& x, W& y, const TwPair<W>& w, const Pr
   }
 }
 
-// inverse butterfly of stage h (h = number of inverse stages already done)
+// kLazy, inverse: slots of one pass whose bits below `stage` are `bits` hold
+// values below 2q 2^lazy_growth after its first `stage` stages (a set bit was
+// a product, below 2q; every clear bit above it a doubling)
+constexpr int lazy_growth(int bits, int stage) {
+  int g = stage;
+  for (int i = 0; i < stage; ++i)
+    if ((bits >> i) & 1) g = stage - 1 - i;
+  return g;
+}
+
+// x below 2q 2^G -> below 2q
+template <int G, typename W>
+__device__ __forceinline__ W lazy_reduce(W x, const PrimeConst<W>& pc) {
+  if constexpr (G == 0)
+    return x;
+  else
+    return lazy_reduce<G - 1>(csub(x, pc.q2 << (G - 1)), pc);
+}
+
+// inverse butterfly of stage h (h = number of inverse stages already done;
+// kLazy: the growth of both slots in this pass)
 template <typename W, int MODE, int H>
 __device__ __forceinline__ void gs_bfly(W& x, W& y, W w, W wp, const PrimeConst<W>& pc) {
-  if constexpr (MODE == kSmall) {
+  if constexpr (MODE == kSmall || MODE == kLazy) {
     W d = x - y + (pc.q << (H + 1));
     x = x + y;
     y = shoup(d, w, wp, pc.q);
@@ -182,7 +209,7 @@ __device__ __forceinline__ void gs_bfly(W& x, W& y, W w, W wp, const PrimeConst<
 template <typename W, int MODE, int H>
 __device__ __forceinline__ void gs_last(W& x, W& y, const PrimeConst<W>& pc) {
   W s, d;
-  if constexpr (MODE == kSmall) {
+  if constexpr (MODE == kSmall || MODE == kLazy) {
     s = x + y;
     d = x - y + (pc.q << (H + 1));
   } else if constexpr (MODE == kL4) {
@@ -233,6 +260,10 @@ __device__ __forceinline__ void fwd_phase(W (&xa)[S::R], W (&xb)[S::R], const Tw
           constexpr int lw = decltype(lwc)::value;
           constexpr int u0 = gl * PB::GS + ((up << (hb + 1)) | lw);
           constexpr int u1 = u0 + (1 << hb);
+          if constexpr (MODE == kLazy && LOGN - 1 - h >= 15) {  // 31q after 15 stages
+            xa[u0] = csub(xa[u0], pc.q2 << 3);
+            if constexpr (TWO) xb[u0] = csub(xb[u0], pc.q2 << 3);
+          }
           ct_bfly<W, MODE>(xa[u0], xa[u1], w, pc);
           if constexpr (TWO) ct_bfly<W, MODE>(xb[u0], xb[u1], w, pc);
         });
@@ -278,8 +309,9 @@ __device__ __forceinline__ void inv_phase_n(W (&x)[S::R], W (&y)[S::R], const Tw
         sfor<0, (1 << hb)>([&](auto lwc) {
           constexpr int lw = decltype(lwc)::value;
           constexpr int u0 = gl * PB::GS + ((up << (hb + 1)) | lw);
-          gs_bfly<W, MODE, h>(x[u0], x[u0 + (1 << hb)], w.w, w.wp, pc);
-          if constexpr (TWO) gs_bfly<W, MODE, h>(y[u0], y[u0 + (1 << hb)], w.w, w.wp, pc);
+          constexpr int hh = MODE == kLazy ? lazy_growth(lw, hb) : h;
+          gs_bfly<W, MODE, hh>(x[u0], x[u0 + (1 << hb)], w.w, w.wp, pc);
+          if constexpr (TWO) gs_bfly<W, MODE, hh>(y[u0], y[u0 + (1 << hb)], w.w, w.wp, pc);
         });
       };
       if constexpr (h == LOGN - 1) {
@@ -288,8 +320,9 @@ __device__ __forceinline__ void inv_phase_n(W (&x)[S::R], W (&y)[S::R], const Tw
           sfor<0, (1 << hb)>([&](auto lwc) {
             constexpr int lw = decltype(lwc)::value;
             constexpr int u0 = gl * PB::GS + ((up << (hb + 1)) | lw);
-            gs_last<W, MODE, h>(x[u0], x[u0 + (1 << hb)], pc);
-            if constexpr (TWO) gs_last<W, MODE, h>(y[u0], y[u0 + (1 << hb)], pc);
+            constexpr int hh = MODE == kLazy ? lazy_growth(lw, hb) : h;
+            gs_last<W, MODE, hh>(x[u0], x[u0 + (1 << hb)], pc);
+            if constexpr (TWO) gs_last<W, MODE, hh>(y[u0], y[u0 + (1 << hb)], pc);
           });
         });
       } else if constexpr (NUP == 1) {
@@ -305,6 +338,14 @@ __device__ __forceinline__ void inv_phase_n(W (&x)[S::R], W (&y)[S::R], const Tw
       }
     });
   });
+  if constexpr (MODE == kLazy && PB::HI < LOGN) {
+    sfor<0, S::R>([&](auto ec) {
+      constexpr int e = decltype(ec)::value;
+      constexpr int g = lazy_growth(e & (PB::GS - 1), PB::B);
+      x[e] = lazy_reduce<g>(x[e], pc);
+      if constexpr (TWO) y[e] = lazy_reduce<g>(y[e], pc);
+    });
+  }
 }
 
 template <class S, int MODE, int P, typename W = typename S::W>
@@ -364,6 +405,15 @@ __device__ __forceinline__ void load_layout(W (&x)[S::R], const CB& s, uint32_t 
     constexpr int e = decltype(ec)::value;
     x[e] = s.load(elem_index<S, P>(e, t));
   });
+}
+
+// kLazy: x, y below 32q from the forward transforms -> x y 2^-64 below 2q.
+// Below 16q each, the Montgomery product is below (256 q / 2^64 + 1) q <= 9q.
+template <typename W>
+__device__ __forceinline__ W lazy_product(W x, W y, const PrimeConst<W>& pc) {
+  const W c16 = pc.q2 << 3;
+  const W u = csub(montmul(csub(x, c16), csub(y, c16), pc.q, pc.qinv), pc.q2 << 2);
+  return lazy_reduce<2>(u, pc);
 }
 
 // ---------------------------------------------------------------- exchanges
@@ -523,6 +573,8 @@ __device__ __forceinline__ void polymul_unit(W* __restrict__ c, const TwPair<W>*
     constexpr int e = decltype(ec)::value;
     if constexpr (MODE == kSmall) {
       xa[e] = montmul(xa[e], xb[e], pc.q, pc.qinv);
+    } else if constexpr (MODE == kLazy) {
+      xa[e] = lazy_product(xa[e], xb[e], pc);
     } else if constexpr (MODE == kL4) {
       xa[e] = csub(montmul(xa[e], xb[e], pc.q, pc.qinv), pc.q2);
     } else {
@@ -585,6 +637,8 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
     const W y = sa[e * S::T + t];
     if constexpr (MODE == kSmall) {
       x[e] = montmul(y, x[e], pc.q, pc.qinv);
+    } else if constexpr (MODE == kLazy) {
+      x[e] = lazy_product(y, x[e], pc);
     } else if constexpr (MODE == kL4) {
       x[e] = csub(montmul(y, x[e], pc.q, pc.qinv), pc.q2);
     } else {

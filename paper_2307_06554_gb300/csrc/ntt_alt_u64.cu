@@ -14,7 +14,7 @@ bool lookup_ntt_alt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
     if (mode == 2) return lookup_ntt_alt_u32_m2(logn, ki);
     return false;
   }
-  if (mode != 1) return false;
+  if (mode != 1 && mode != 4) return false;  // the Harvey-bound kernels hold for both
   switch (logn) {
 #define PM_R16(L)                                                   \
   case L:                                                           \

@@ -301,6 +301,8 @@ template <class S, int MODE, typename W = typename S::W>
 __device__ __forceinline__ W pointwise1(W x, W y, const PrimeConst<W>& pc) {
   if constexpr (MODE == kSmall) {
     return montmul(x, y, pc.q, pc.qinv);
+  } else if constexpr (MODE == kLazy) {
+    return lazy_product(x, y, pc);
   } else if constexpr (MODE == kL4) {
     return csub(montmul(x, y, pc.q, pc.qinv), pc.q2);
   } else {
@@ -443,6 +445,9 @@ bool lookup_ntt_cluster2(uint32_t elem, int logn, int mode, bool seq, KernelInfo
     PM_C2(uint64_t, 14, 1, 4, 13, 128)
     PM_C2(uint64_t, 15, 1, 4, 13, 128)
     PM_C2(uint64_t, 16, 1, 4, 13, 128)
+    PM_C2(uint64_t, 14, kLazy, 4, 13, 128)
+    PM_C2(uint64_t, 15, kLazy, 4, 13, 128)
+    PM_C2(uint64_t, 16, kLazy, 4, 13, 128)
   } else {
     PM_C2(uint32_t, 14, 0, 4, 13, 128)
     PM_C2(uint32_t, 15, 0, 4, 12, 64)
@@ -470,6 +475,9 @@ bool lookup_ntt_cluster_small(uint32_t elem, int logn, int mode, KernelInfo* ki)
     PM_CS(uint64_t, 13, 1, 3, 12)
     PM_CS(uint64_t, 14, 1, 3, 12)
     PM_CS(uint64_t, 15, 1, 3, 12)
+    PM_CS(uint64_t, 13, kLazy, 3, 12)
+    PM_CS(uint64_t, 14, kLazy, 3, 12)
+    PM_CS(uint64_t, 15, kLazy, 3, 12)
   } else {
     PM_CS(uint32_t, 14, 0, 4, 12)
     PM_CS(uint32_t, 14, 1, 4, 12)

@@ -101,13 +101,15 @@ inline void build_tiny_tables(uint64_t q, uint32_t n, std::vector<uint32_t>& twf
 }
 
 // Reduction mode for the largest modulus (see the mode notes in ntt.cuh):
-// 2 = no conditional subtractions, 1 = Harvey [0, 4q), 0 = [0, 2q).
+// 2 = no conditional subtractions, 4 = few of them (64-bit words), 1 = Harvey
+// [0, 4q), 0 = [0, 2q).
 inline int ntt_mode(uint64_t qmax, uint32_t logn, uint32_t elem) {
   using pm::host::u128;
   const int bits = 8 * (int)elem;
   const u128 lim = (u128)1 << bits;
   const u128 g = 1 + 2 * (u128)logn;
   if (((u128)qmax << (logn + 1)) < lim && g * g * qmax < lim) return 2;
+  if (elem == 8 && qmax < (1ull << 59)) return 4;
   if ((u128)qmax * 4 < lim) return 1;
   if ((u128)qmax * 2 < lim) return 0;
   return -1;

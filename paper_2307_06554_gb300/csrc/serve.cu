@@ -652,10 +652,14 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
     return bail(cuda_fail(cudaGetLastError(), "table upload"));
   s->arena_bytes = device_bytes;
   s->free_list[0] = device_bytes;
-  // kernels per degree (64-bit words, Harvey bounds: every pool prime < 2^62)
+  // kernels per degree (64-bit words; Harvey bounds unless every pool prime
+  // is below 2^59)
+  const int mode = *std::max_element(s->pool.begin(), s->pool.end()) < (1ull << 59) ? 4 : 1;
   for (int logn = 4; logn <= (int)s->lognmax; ++logn) {
     KernelInfo ki;
-    const bool ok = logn >= 14 ? lookup_ntt_cluster2(8, logn, 1, false, &ki) : lookup_ntt_u64_m1(logn, &ki);
+    const bool ok = logn >= 14 ? lookup_ntt_cluster2(8, logn, mode, false, &ki)
+                    : mode == 4 ? lookup_ntt_u64_m4(logn, &ki)
+                                : lookup_ntt_u64_m1(logn, &ki);
     if (!ok) return bail(fail(POLYMUL_ENOTSUP, "no kernel for n=2^%d", logn));
     if (ki.smem > 48 * 1024 &&
         cudaFuncSetAttribute(ki.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, ki.smem) != cudaSuccess)
@@ -678,7 +682,7 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
     s->dki[logn] = ki;  // the cluster kernels read and write with plain accesses
     s->dgrid_cap[logn] = cap;
     KernelInfo dk;
-    if (lookup_ntt_cluster_small(8, logn, 1, &dk)) {
+    if (lookup_ntt_cluster_small(8, logn, logn == 12 ? 1 : mode, &dk)) {
       // n = 2^12 .. 2^15: a request is a few rows, so one row's latency is
       // its service time and the lanes' throughput (200 requests of 2^12 ..
       // 2^14, up to 8 primes, 8 lanes, all queued: 1.49 ms with the batch
