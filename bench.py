@@ -1543,6 +1543,10 @@ def run_ours(args, ws, rank, local):
                     "pointwise); the kernel also scales half of the outputs by n^-1: with those, frac %.3f" % (
                         mulmods_kernel / (launch_ms / 1e3) / 1e9 / alu_peak),
             "kernel": tag + " (forward x2, pointwise, inverse; one launch per step)",
+            "note": None if (info["radix_bits"], info["exchange_pad"]) != (5, 3) else
+                    "achieved counts the modular multiplications of a complete transform; this kernel (the unit of "
+                    "the smallest moduli) multiplies by Plantard's method, two low products each, and stops its "
+                    "transforms at eight coefficients, so the Shoup peak is a yardstick, not its ceiling",
             "peak_source": "derived: %d SMs x %d IMAD lanes x %.0f MHz / %d IMAD slots per Shoup mulmod" % (
                 sms, IMAD_LANES_PER_SM, sm_mhz, slots),
             "mulmods_per_launch": mulmods, "launch_ms": launch_ms,

@@ -10,9 +10,9 @@
 // products: 4 % of the forward work) and saves a launch, its scratch and the
 // trip of a^ through memory.  A warp owns two row buffers: the next product's
 // row arrives in one while the other serves this one's exchanges.
-// n = 1024, q = 12289, 4096 products: 25.2 us in two launches, see the
-// kernel's measured time in the commit that brought it and in the design
-// notes; bound by the multiply and add pipes like the batch kernel.
+// n = 1024, q = 12289, 4096 products: 15.0 us, 25.4 in two launches of the
+// general form; bound by issue slots and instruction fetch like the batch
+// kernel, with a fill and a drain per call.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
