@@ -481,8 +481,9 @@ int polymul_ragged_status(polymul_ragged_batch *batch, void *stream);
  * (degrees 2^10 .. 2^13; 2^14) exists in two shape sets -- 0: swizzled
  * exchanges, both operands in registers (2^14: the batch kernel, the
  * default there); 1: padded exchanges at half the registers (the default
- * for 2^10 .. 2^13; 2^14: one operand in registers at a time) -- and each
- * launch keeps the faster set; then each degree class runs on the path that is
+ * for 2^10 .. 2^13, where lists of up to 13000 coefficients per SM take set
+ * 0; 2^14: one operand in registers at a time) -- and each launch keeps the
+ * faster set; then each degree class runs on the path that is
  * faster for its rows: its NTT segment alone, or the tensor path (Sec. 2.2
  * matrix form: the tiled digit kernel with 8-bit digits drained per K
  * chunk, one launch per class, behind the NTT launches).  Best of three
@@ -498,7 +499,7 @@ int polymul_ragged_tune(polymul_ragged_batch *batch, const void *a, const void *
 
 /* Use the shape sets and paths `choice` (bits as for polymul_ragged_tune;
  * tensor bits of classes the list does not hold are ignored) instead of the
- * default (every class on the NTT path, sets 1 and 0) or tuned ones.  Waits for
+ * default (every class on the NTT path, sets as above) or tuned ones.  Waits for
  * the device to finish its work first (the NTT launches' segment list is
  * rewritten).  Errors: EINVAL (choice >= 128, or a class with units and no
  * tensor kernel for the pool: each pool prime needs at most four 8-bit

@@ -69,8 +69,9 @@ struct polymul_ragged_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraphNode_t node[2] = {nullptr, nullptr};
-  // shape set of each launch: the padded set for 2^10 .. 2^13, the batch
-  // kernel for 2^14 by default; polymul_ragged_tune measures both
+  // shape set of each launch: the padded set for 2^10 .. 2^13 (short lists:
+  // set 0, see polymul_ragged_prepare), the batch kernel for 2^14 by default;
+  // polymul_ragged_tune measures both
   int set[2] = {1, 0};
   // degree segments of the whole list (host copy; d_items holds those the
   // NTT launches take), and the classes on the tensor path (bit logn - 10)
@@ -380,6 +381,15 @@ extern "C" int polymul_ragged_prepare(polymul_ragged* r, const polymul_desc* des
   }
   b->items_h = items;
   for (const RaggedItem& it : items) b->present |= 1u << (it.logn - 10);
+  // Short lists take set 0 for the smaller degrees: with one or two units per
+  // team a unit's latency decides, and the 64-register body of set 1 is the
+  // longer one (483 rows of 2^10: 14.7 us against 20.0; 287 rows of 2^11 ..
+  // 2^14 30.3 / 33.2; 448 rows of 2^12, 2^13, 2.7 M coefficients, 39.3 / 38.2;
+  // 3119 rows, 15 M coefficients, 174 / 142).
+  uint64_t small_coeffs = 0;
+  for (const RaggedItem& it : items)
+    if (it.logn < 14) small_coeffs += (uint64_t)it.count << it.logn;
+  if (small_coeffs <= 13000ull * (uint64_t)r->num_sms) b->set[0] = 0;
   apply_paths(b);
   *out = b;
   return POLYMUL_OK;
