@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "host_math.h"
+#include "ntt_tiny_arith.h"
 #include "polymul_types.h"
 
 namespace pm {
@@ -64,15 +65,8 @@ inline void build_ntt_tables(uint64_t q, uint32_t n, std::vector<W>& twf, std::v
 // Tables of the unit for the smallest moduli (ntt_tiny.cuh): n / 8 words
 // forward and n / 8 inverse (entry k as in build_ntt_tables_into, k < n / 8;
 // the transform stops at polynomials of 8 coefficients, so a root of order
-// 2n / 8, n / 8 for the cyclic ring, is enough), each the word
-// (-w 2^32 mod q, centred) q^-1 mod 2^32 of a root w, and the constants the
-// unit reads from PrimeConst.
-constexpr uint32_t kTinyQMax = 18500;  // exclusive
-inline uint32_t tiny_word(uint64_t w, uint64_t q) {
-  const int64_t W = (int64_t)((q - w % q * ((1ull << 32) % q) % q) % q);
-  const int64_t centred = W > (int64_t)(q / 2) ? W - (int64_t)q : W;
-  return (uint32_t)((uint64_t)centred * pm::host::inv_pow2_64(q));
-}
+// 2n / 8, n / 8 for the cyclic ring, is enough), each the word of a root
+// (tiny_word), and the constants the unit reads from PrimeConst.
 inline void build_tiny_tables(uint64_t q, uint32_t n, std::vector<uint32_t>& twf, std::vector<uint32_t>& twi,
                               PrimeConst<uint32_t>& pc, bool cyclic = false) {
   using namespace pm::host;

@@ -3,18 +3,12 @@
 //
 // Two things set it apart from polymul_unit (ntt.cuh):
 //
-//  * Plantard's multiplication by a constant in 32-bit words (T. Plantard,
-//    "Efficient word size modular arithmetic", 2021; the signed form for
-//    small moduli of Huang et al., "Improved Plantard arithmetic for
-//    lattice-based cryptography", 2022).  With q' = q^-1 mod 2^32 and W the
-//    centred residue of -w 2^32, let z = a (W q') mod 2^32 (signed); then
-//    z q - a W is a multiple of 2^32 and its quotient k is congruent to a w.
-//    k = floor(((z >> 16) q + 2^15) / 2^16) whenever |a W| <= 2^31 - 2^15 q,
-//    and |k| <= (q + 1) / 2.  One precomputed word per root, two low
-//    products, two shifts (the second fused with the butterfly's addition):
-//    23.5 butterflies per SM per clock measured, against 13 for the Shoup
-//    form of ntt.cuh (whose high product takes two issue slots of the
-//    multiply pipe).  No reduction is needed on the way forward.
+//  * Plantard's multiplication by a constant (ntt_tiny_arith.h): one
+//    precomputed word per root, two low products, two shifts (the second
+//    fused with the butterfly's addition): 23.5 butterflies per SM per clock
+//    measured, against 13 for the Shoup form of ntt.cuh (whose high product
+//    takes two issue slots of the multiply pipe).  No reduction is needed on
+//    the way forward.
 //  * The transform stops at polynomials of 8 coefficients: the ring splits
 //    into n / 8 rings x^8 - z, and the products there are 64 multiply-adds
 //    of centred residues whose sums of eight fit 32 bits, reduced once per
@@ -31,36 +25,18 @@
 // of the top layout and 16-byte accesses of the low one are both free of
 // bank conflicts.
 //
-// Bounds, in units of q / 2: inputs 2, one more per forward stage (at most
-// 9); b is brought back to 1 before the products, a when it is parked.  The
-// inverse doubles per stage without a multiplication; tiny_bounds tracks it
-// slot by slot at compile time and reduces a slot where a sum could pass
-// kTinyLim (q < 18500 keeps kTinyLim q^2 / 4 below 2^31 - 2^15 q).
+// Bounds, in units of (q - 1) / 2: inputs 2, one more per forward stage (at
+// most 9); b is brought back to 1 before the products, a when it is parked.
+// The inverse doubles per stage without a multiplication; tiny_bounds tracks
+// it slot by slot at compile time and reduces a slot where a sum could pass
+// kTinyLim, the largest factor the multiplication takes.
 #pragma once
 #include <cstdint>
 
 #include "arith.cuh"
+#include "ntt_tiny_arith.h"
 
 namespace pm {
-
-constexpr int kTinyLogM = 3;                // coefficients per remaining ring
-constexpr int kTinyM = 1 << kTinyLogM;
-constexpr int kTinyLim = 18;                // largest factor of a product, in units of q / 2 (q < kTinyQMax)
-
-struct TinyMod {
-  int q, qinv;  // the prime, q^-1 mod 2^32
-};
-
-// z = a (W q') mod 2^32 -> a w mod q in [-(q+1)/2, (q+1)/2], before the last shift
-__device__ __forceinline__ int tiny_pre(int z, const TinyMod& m) { return (z >> 16) * m.q + 32768; }
-__device__ __forceinline__ int tiny_mul(int a, int w, const TinyMod& m) { return tiny_pre(a * w, m) >> 16; }
-
-// x, y -> x + w y, x - w y
-__device__ __forceinline__ void tiny_ct(int& x, int& y, int w, const TinyMod& m) {
-  const int s = x + (tiny_pre(y * w, m) >> 16);
-  y = 2 * x - s;
-  x = s;
-}
 
 // Compile-time bounds of the inverse stages on 32 slots.
 struct TinyBounds {
@@ -209,7 +185,7 @@ __device__ __forceinline__ void tiny_forward(int (&x)[32], const uint32_t* in, i
   tiny_fwd_low<S>(x, tw, m, t);
 }
 
-// c = a b in the ring x^8 - z: a, b within (q + 1) / 2, wz the root's word
+// c = a b in the ring x^8 - z: a, b within (q - 1) / 2, wz the root's word
 __device__ __forceinline__ void tiny_ring(int* b, const int (&a)[8], int wz, const TinyMod& m) {
   int az[8];
   sfor<1, 8>([&](auto ic) {
@@ -333,7 +309,7 @@ __device__ __forceinline__ void tiny_finish(uint32_t* __restrict__ c, int (&x)[3
   if (act) {
     sfor<0, 32>([&](auto ec) {
       constexpr int e = decltype(ec)::value;
-      // [-(q+1)/2, (q+1)/2] -> [0, q): as unsigned words the negative ones are the larger
+      // [-(q-1)/2, (q-1)/2] -> [0, q): as unsigned words the negative ones are the larger
       c[t + TS::T * e] = __viaddmin_u32((uint32_t)x[e], pc.q, (uint32_t)x[e]);
     });
   }
