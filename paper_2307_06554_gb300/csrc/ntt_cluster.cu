@@ -44,6 +44,15 @@ struct ClusterSync {
   }
 };
 
+// The first barrier of a cluster kernel.  The CTAs of a cluster need not
+// start together, and the shared memory of one that has not started may not
+// be accessed: every CTA arrives on entry and waits before its first unit.
+// (Waiting behind the first unit's loads, inside the loop, hides the barrier
+// but costs the 64-bit kernels more in the loop: 128 products at 2^15 182.8
+// us so, 188.2 inside.)
+__device__ __forceinline__ void cluster_start_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_start_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -106,6 +115,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster(NttBatchArgs
   using Buf = ClusterBuf<W, S::RB, kClusterLocalLog>;
   static_assert(S::T % kClusterThreads == 0 && S::N == (S::T / kClusterThreads) << kClusterLocalLog,
                 "one CTA per 8192 coefficients");
+  cluster_start_arrive();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   W* buf = reinterpret_cast<W*>(smem_raw);
   constexpr uint32_t L = 1u << kClusterLocalLog;
@@ -117,6 +127,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1) k_ntt_cluster(NttBatchArgs
   constexpr int TOP = S::NPH - 1;
   const TwPair<W>* twf = reinterpret_cast<const TwPair<W>*>(args.tw_fwd);
   const TwPair<W>* twi = reinterpret_cast<const TwPair<W>*>(args.tw_inv);
+  cluster_start_wait();
   for (uint64_t u = cluster_id(); u < args.units; u += cluster_count()) {
     const uint32_t j = (uint32_t)(u % args.k);
     const uint32_t pj = table_index(args, j);
@@ -270,7 +281,8 @@ __device__ __forceinline__ void cmid() {
 // Before the stores of an exchange nothing is needed: a local layout is
 // stored at the positions this thread loaded, and the top layout's remote
 // stores follow a cluster barrier that every CTA passed after its last
-// access to the buffer (see k_ntt_cluster2).
+// access to the buffer (see k_ntt_cluster2; the first unit's follow
+// cluster_start_wait).
 template <class S, int MODE, int P, bool TWO, typename W = typename S::W>
 __device__ __forceinline__ void cfwd(W (&xa)[S::R], W (&xb)[S::R], W* sa, W* sb, const TwPair<W>* __restrict__ tw,
                                      const PrimeConst<W>& pc, uint32_t t) {
@@ -324,6 +336,7 @@ __global__ void __launch_bounds__(S::CT, 65536 / (S::CT * REGS)) k_ntt_cluster2(
   static_assert(S::PAD > 0, "padded local layout");
   static_assert(!cta_local<S, S::NPH - 1>(), "the top layout spans the cluster");
   static_assert(cta_local<S, S::NPH - 2>(), "every other layout is local to a CTA (see cstore)");
+  cluster_start_arrive();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr uint32_t L = (1u << S::LL) + ((1u << S::LL) >> S::PAD);
   W* sa = reinterpret_cast<W*>(smem_raw);
@@ -333,6 +346,7 @@ __global__ void __launch_bounds__(S::CT, 65536 / (S::CT * REGS)) k_ntt_cluster2(
   const TwPair<W>* twf = reinterpret_cast<const TwPair<W>*>(args.tw_fwd);
   const TwPair<W>* twi = reinterpret_cast<const TwPair<W>*>(args.tw_inv);
   const W* g0 = nullptr;
+  cluster_start_wait();
   for (uint64_t u = cluster_id(); u < args.units; u += cluster_count()) {
     const uint32_t j = (uint32_t)(u % args.k);
     const uint32_t pj = table_index(args, j);
