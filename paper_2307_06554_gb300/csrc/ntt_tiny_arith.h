@@ -58,11 +58,13 @@ struct TinyMod {
 
 // z = a (W q') mod 2^32 -> a w mod q in [-(q-1)/2, (q-1)/2], before the last shift
 PM_HD int tiny_pre(int z, const TinyMod& m) { return (z >> 16) * m.q + kTinyRound; }
-PM_HD int tiny_mul(int a, int w, const TinyMod& m) { return tiny_pre(a * w, m) >> 16; }
+// the low product wraps: unsigned, where that is defined
+PM_HD int tiny_low(int a, int w) { return (int)((uint32_t)a * (uint32_t)w); }
+PM_HD int tiny_mul(int a, int w, const TinyMod& m) { return tiny_pre(tiny_low(a, w), m) >> 16; }
 
 // x, y -> x + w y, x - w y
 PM_HD void tiny_ct(int& x, int& y, int w, const TinyMod& m) {
-  const int s = x + (tiny_pre(y * w, m) >> 16);
+  const int s = x + tiny_mul(y, w, m);
   y = 2 * x - s;
   x = s;
 }

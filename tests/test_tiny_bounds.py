@@ -74,6 +74,14 @@ def test_multiplication_over_its_range(tmp_path):
     assert r.returncode == 0, r.stdout
 
 
+def test_no_signed_overflow(tmp_path):
+    """The low product wraps in unsigned arithmetic: built with traps on signed
+    overflow, the same range runs through."""
+    exe = build_host(tmp_path, ["-fsanitize=signed-integer-overflow", "-fsanitize-undefined-trap-on-error"])
+    r = subprocess.run([exe, "7681", "12289", "18433"], capture_output=True, text=True)
+    assert r.returncode == 0, (r.returncode, r.stdout)
+
+
 def _root(q, order):
     """The library's root: the smallest base whose power has exactly this order."""
     for g in range(2, q):
