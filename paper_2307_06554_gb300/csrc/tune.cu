@@ -6,7 +6,8 @@
 // operand, and the tensor path where the shape allows it) runs on a batch
 // of the requested size, and the fastest is kept.  Results are cached per
 // (GPU, word, n, k, mode, modulus bits, batch bucket) in the process and,
-// if POLYMUL_TUNE_CACHE names a file, on disk as "key<TAB>label" lines.
+// if POLYMUL_TUNE_CACHE names a file, on disk as "key<TAB>label" lines; a
+// stored label that names none of the plan's candidates is measured again.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -58,10 +59,22 @@ void store_cache(const std::string& key, const std::string& label) {
   f << key << '\t' << label << '\n';
 }
 
+// Names one candidate of a plan, across processes: everything that tells its
+// kernels apart (two shapes of one radix, or two cluster sizes, would share a
+// shorter label, and a stored choice would come back as the other kernel).
 std::string label_of(const PlanCandidate& c) {
-  if (c.path == POLYMUL_PATH_TENSOR) return c.ki.rns ? "tensor-rns" : c.ki.tiled ? "tensor-tiled" : "tensor";
-  if (c.ki.tiny) return "ntt-tiny";
-  return "ntt-rb" + std::to_string(c.ki.rb) + (c.ki.cluster ? "-cluster" : "");
+  const KernelInfo& k = c.ki;
+  char buf[96];
+  if (c.path == POLYMUL_PATH_TENSOR)
+    snprintf(buf, sizeof buf, "tensor-%s%s%s-w%d-d%d-b%d-t%d-s%d",
+             k.rns     ? "rns"
+             : k.u64   ? "u64"
+             : k.tiled ? "tiled"
+                       : "whole",
+             k.drain ? "-drain" : "", k.ws ? "-ws" : "", k.wb, k.digits, k.block, k.tmem_cols, k.smem);
+  else
+    snprintf(buf, sizeof buf, "ntt-rb%d-m%d-r%d-p%d-o%d-b%d-s%d", k.rb, k.mode, k.regs, k.pad, k.seq, k.block, k.smem);
+  return buf;
 }
 
 uint64_t bucket_of(uint64_t batch) {
