@@ -113,6 +113,8 @@ typedef struct polymul_opts {
     uint32_t reserved[5];
 } polymul_opts;
 
+/* "Main kernel": the plan's chosen candidate (see polymul_batch for the
+ * kernel of small batches). */
 typedef struct polymul_plan_info {
     uint32_t n;
     uint32_t k;
@@ -134,7 +136,9 @@ typedef struct polymul_plan_info {
                              kernel on the stream drains and wait for it to
                              complete before touching memory); set for the
                              NTT batch kernels.  Bit 2: POLYMUL_FLAG_OVERLAP
-                             is in effect for it                            */
+                             is in effect for it (a small batch may run a
+                             thread-block-cluster kernel, which waits for its
+                             predecessor: see polymul_batch)                */
     uint32_t ntt_mode;    /* NTT path: reduction mode of the main kernel:
                              0 = values in [0, 2q), 1 = [0, 4q) (Harvey),
                              2 = unreduced (small q), 4 = 64-bit words
@@ -207,6 +211,10 @@ int polymul_create(uint32_t n, const uint64_t *q_list, uint32_t k,
  *   a, b, c  device pointers, [batch][k][n] of the plan's element type,
  *            16-byte aligned.  batch == 0 is a no-op.
  *   stream   cudaStream_t or NULL.
+ * A plan whose kernel has not been tuned or selected may run another of its
+ * candidates for a batch too small to fill the GPU, with more threads per
+ * product; results are the same, and polymul_plan_info describes the kernel
+ * of the larger batches.
  * Asynchronous.  The tensor path's residue-number-system kernel keeps
  * residue planes in plan-owned scratch, allocated (or grown) on the first
  * call with a larger batch: make one such call before capturing the stream
@@ -354,7 +362,9 @@ int polymul_static_status(void *stream);
  * cached per (GPU, word size, n, k, reduction mode, modulus size, batch
  * bucket) for the process, and in the file named by the environment
  * variable POLYMUL_TUNE_CACHE if set (read on first use, appended after each
- * new measurement).  Allocates scratch buffers for the measurement only.
+ * new measurement).  A tuned plan runs the kept kernel for every batch size,
+ * except that the default kernel, when it is kept, keeps the other kernel
+ * that smaller batches take without tuning (see polymul_batch).  Allocates scratch buffers for the measurement only.
  * Synchronous.  Errors: EINVAL, ENOMEM, ECUDA.
  */
 int polymul_tune(polymul_plan *plan, uint64_t batch, void *stream);
@@ -407,7 +417,8 @@ int polymul_tensor_shape(uint32_t n, uint64_t qmax, uint32_t flags, polymul_tens
 int polymul_tensor_rns_base(uint32_t n, uint64_t qmax, uint32_t *moduli, uint32_t cap, uint32_t *count);
 
 /* Use candidate kernel `candidate` (0 .. info.candidates - 1; 0 is the
- * default) instead of the tuned or default choice.  Errors: EINVAL. */
+ * default) instead of the tuned or default choice, whatever the batch (see
+ * polymul_batch).  Errors: EINVAL. */
 int polymul_plan_select(polymul_plan *plan, uint32_t candidate);
 
 /* Fill *info with the plan's shape and launch configuration. */

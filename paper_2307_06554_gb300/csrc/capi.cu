@@ -569,9 +569,9 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     p->small = few;
     const uint64_t sms = (uint64_t)p->num_sms;
     if (p->elem == 8)
-      p->small_units = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
+      p->small_line = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
     else
-      p->small_units = p->logn == 14 ? sms / 2 : p->logn == 13 ? sms : sms * 2048 / p->n;
+      p->small_line = p->logn == 14 ? sms / 2 : p->logn == 13 ? sms : sms * 2048 / p->n;
   }
   // Small batches leave most of the GPU idle whatever the kernel: one unit's
   // latency is the call, and more threads per unit with shorter chains win.
@@ -585,9 +585,10 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     const bool aux2 = p->aux_prime != 0;
     if (aux2 || p->cands[0].ki.tiny) {
       p->small = 1;
-      p->small_units = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
+      p->small_line = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
     }
   }
+  p->small_units = p->small_line;
   if (rc == POLYMUL_OK) {
     // work counters for the three launch slots (device entry, two host-entry streams)
     if (cudaMalloc(&p->d_ctr, 2 * kCounterSlots * sizeof(unsigned long long)) != cudaSuccess ||

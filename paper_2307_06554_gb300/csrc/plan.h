@@ -48,10 +48,12 @@ struct polymul_plan {
   pm::KernelInfo tki;  // tensor-path kernel, when one exists for the shape
   std::vector<PlanCandidate> cands;  // [0] is the default
   size_t chosen = 0;
-  // batches of at most small_units units run candidate `small` instead, as
-  // long as the choice is the default one (see polymul_create); 0: none
+  // batches of at most small_units units run candidate `small` instead of
+  // the default one (see polymul_create); 0: none.  small_line is that limit
+  // as created: small_units is 0 while another candidate, or explicitly the
+  // default one (polymul_plan_select), is chosen
   size_t small = 0;
-  uint64_t small_units = 0;
+  uint64_t small_units = 0, small_line = 0;
   bool tuned = false;
   uint64_t tuned_batch = 0;  // batch bucket of the tuned choice
   void* d_tpc = nullptr;  // tensor-path constants

@@ -77,6 +77,15 @@ std::string label_of(const PlanCandidate& c) {
   return buf;
 }
 
+// The tuned choice.  The default candidate keeps its form for small batches,
+// unless it was measured at such a batch and won there.
+void settle(polymul_plan* p, size_t i, uint64_t bucket) {
+  apply_candidate(p, i);
+  if (i == 0 && bucket * p->k > p->small_line) p->small_units = p->small_line;
+  p->tuned = true;
+  p->tuned_batch = bucket;
+}
+
 uint64_t bucket_of(uint64_t batch) {
   uint64_t b = 1;
   while (b < batch && b < (1ull << 16)) b <<= 1;
@@ -112,9 +121,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
   if (hit != g_tune_cache.end()) {
     for (size_t i = 0; i < p->cands.size(); ++i)
       if (label_of(p->cands[i]) == hit->second) {
-        apply_candidate(p, i);
-        p->tuned = true;
-        p->tuned_batch = bucket;
+        settle(p, i, bucket);
         return POLYMUL_OK;
       }
   }
@@ -138,6 +145,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
       cudaEventCreate(&e1) != cudaSuccess)
     rc = fail(POLYMUL_ECUDA, "tuning setup failed");
   const size_t saved_chosen = p->chosen;
+  const uint64_t saved_small = p->small_units;
   const uint32_t saved_flags = p->flags;
   p->flags &= ~POLYMUL_FLAG_VALIDATE;
   std::vector<float> best_ms(p->cands.size(), 1e30f);
@@ -186,10 +194,12 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(buf);
-  apply_candidate(p, rc == POLYMUL_OK ? best : saved_chosen);
-  if (rc != POLYMUL_OK) return rc;
-  p->tuned = true;
-  p->tuned_batch = bucket;
+  if (rc != POLYMUL_OK) {
+    apply_candidate(p, saved_chosen);
+    p->small_units = saved_small;
+    return rc;
+  }
+  settle(p, best, bucket);
   store_cache(key, label_of(p->cands[best]));
   return POLYMUL_OK;
 }
