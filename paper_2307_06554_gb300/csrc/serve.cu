@@ -43,6 +43,7 @@
 #include "kernels.h"
 #include "trace.h"
 #include "plan.h"
+#include "serve_queue.h"
 #include "polymul_types.h"
 
 using namespace pm;
@@ -113,14 +114,8 @@ struct polymul_server {
   // streams of their own joined by events, so that a request's copies in do
   // not wait for the previous request's kernel and copy out on the lane
   std::vector<cudaStream_t> lanes, lanes_in, lanes_out;
-  // A direct request is one kernel, so it needs one stream, not a pipeline:
-  // it may take any of a lane's three.  Queue q: 0 .. nlanes - 1 the kernel
-  // streams (a staged request's lane is the queue of its kernel), then the
-  // copy-in, then the copy-out streams.  A request's kernel spends most of
-  // its time waiting for the host link, so three times as many of them in
-  // flight keep the link busier (200 requests of 2^12 .. 2^14, up to 8
-  // primes, 8 lanes: 1.23 ms on the kernel streams alone, 1.10 with the others).
-  int direct_queues() const { return 3 * nlanes; }
+  // the three streams of every lane as queues, with the load of each
+  ServeQueues queues;
   cudaStream_t queue_stream(int q) const {
     return q < nlanes ? lanes[q] : q < 2 * nlanes ? lanes_in[q - nlanes] : lanes_out[q - 2 * nlanes];
   }
@@ -160,7 +155,6 @@ struct polymul_server {
   std::vector<std::deque<ServeReq*>> lane_fifo;
   size_t inflight = 0;
   std::vector<cudaEvent_t> event_pool;
-  std::vector<uint64_t> lane_bytes;  // bytes of the requests in flight on each lane
   std::atomic<bool> stop{false};
   std::thread loop;
   int cuda_error = 0;
@@ -407,9 +401,9 @@ void server_loop(polymul_server* s) {
     // retire: only the oldest request of each queue can be the next to
     // finish; at most as many queues per pass as there are lanes, in turn, so
     // that the event queries of a pass between two admissions stay few
-    for (int i = 0, looked = 0; i < s->direct_queues() && looked < s->nlanes; ++i) {
+    for (int i = 0, looked = 0; i < s->queues.queues() && looked < s->nlanes; ++i) {
       std::deque<ServeReq*>& f = s->lane_fifo[scan];
-      scan = scan + 1 == s->direct_queues() ? 0 : scan + 1;
+      scan = scan + 1 == s->queues.queues() ? 0 : scan + 1;
       if (!f.empty()) ++looked;
       while (!f.empty()) {
         ServeReq* r = f.front();
@@ -427,7 +421,7 @@ void server_loop(polymul_server* s) {
         s->free_slots.push_back(r->slot);
         r->slot = -1;
         if (r->bytes) arena_free(s, r->off, r->bytes);
-        s->lane_bytes[r->lane] -= r->weight;
+        s->queues.release(r->lane, r->direct, r->weight);
         release_events(s, r);
         f.pop_front();
         --s->inflight;
@@ -440,20 +434,7 @@ void server_loop(polymul_server* s) {
       const size_t off = r->bytes ? arena_alloc(s, r->bytes) : 0;  // a direct request may need none
       if (off == (size_t)-1) break;
       r->off = off;
-      // the lane with the least work in flight: a small request does not
-      // queue behind a large one while another lane is idle
-      int lane = 0;
-      for (int l = 1; l < s->nlanes; ++l)
-        if (s->lane_bytes[l] < s->lane_bytes[lane]) lane = l;
-      // A direct request that moves half a MB or more finds another queue
-      // when every lane is busy.  Smaller ones keep to the lanes: there the
-      // server thread's issue time is the bound, and launches on more streams
-      // cost it more (1000 requests of 2^10 .. 2^12: 4.4 -> 4.7 us each).
-      if (r->direct && r->weight >= (512u << 10) && s->lane_bytes[lane] > 0)
-        for (int l = s->nlanes; l < s->direct_queues(); ++l)
-          if (s->lane_bytes[l] < s->lane_bytes[lane]) lane = l;
-      r->lane = lane;
-      s->lane_bytes[lane] += r->weight;
+      r->lane = s->queues.admit(r->direct, r->weight);
       take_events(s, r);
       r->slot = s->free_slots.back();  // fewer than max_inflight requests are in flight
       s->free_slots.pop_back();
@@ -471,11 +452,11 @@ void server_loop(polymul_server* s) {
         s->free_slots.push_back(r->slot);
         r->slot = -1;
         if (r->bytes) arena_free(s, r->off, r->bytes);
-        s->lane_bytes[r->lane] -= r->weight;
+        s->queues.release(r->lane, r->direct, r->weight);
         release_events(s, r);
         done.push_back(r);
       } else {
-        s->lane_fifo[lane].push_back(r);
+        s->lane_fifo[r->lane].push_back(r);
         ++s->inflight;
       }
       progress = true;
@@ -607,8 +588,8 @@ extern "C" int polymul_server_create(const uint64_t* pool, uint32_t pool_size, u
   s->lognmax = __builtin_ctz(n_max);
   s->pool.assign(pool, pool + pool_size);
   s->nlanes = (int)lanes;
-  const size_t queues = (size_t)s->direct_queues();
-  s->lane_bytes.assign(queues, 0);
+  s->queues.reset((int)lanes);
+  const size_t queues = (size_t)s->queues.queues();
   s->lane_fifo.resize(queues);
   s->max_inflight = std::max<size_t>(64, 8 * (size_t)lanes);  // enough requests to keep every lane busy
   int rc = POLYMUL_OK;
