@@ -401,9 +401,10 @@ void server_loop(polymul_server* s) {
     // retire: only the oldest request of each queue can be the next to
     // finish; at most as many queues per pass as there are lanes, in turn, so
     // that the event queries of a pass between two admissions stay few
-    for (int i = 0, looked = 0; i < s->queues.queues() && looked < s->nlanes; ++i) {
-      std::deque<ServeReq*>& f = s->lane_fifo[scan];
-      scan = scan + 1 == s->queues.queues() ? 0 : scan + 1;
+    const int occupied = s->queues.occupied();
+    for (int i = 0, looked = 0; i < occupied && looked < s->nlanes; ++i) {
+      if (scan >= occupied) scan = 0;
+      std::deque<ServeReq*>& f = s->lane_fifo[scan++];
       if (!f.empty()) ++looked;
       while (!f.empty()) {
         ServeReq* r = f.front();

@@ -18,11 +18,16 @@ class ServeQueues {
  public:
   void reset(int lanes) {
     lanes_ = lanes;
+    beyond_ = 0;
     load_.assign((size_t)3 * lanes, 0);
   }
   int lanes() const { return lanes_; }
   int queues() const { return 3 * lanes_; }
   uint64_t load(int q) const { return load_[q]; }
+  // the queues that may hold requests: past the lanes only while a direct
+  // request is on one of them (24 empty queues looked at on every pass cost
+  // the server thread 1 % of a request's 4.4 us)
+  int occupied() const { return beyond_ ? queues() : lanes_; }
 
   // The queue of a request that moves `weight` bytes, charged with them (a
   // staged request's queue is the kernel stream of its lane).
@@ -37,6 +42,7 @@ class ServeQueues {
  private:
   void add(int q, bool direct, int64_t w) {
     load_[q] += (uint64_t)w;
+    if (q >= lanes_) beyond_ += w < 0 ? -1 : 1;
     if (!direct) {
       load_[lanes_ + q] += (uint64_t)w;
       load_[2 * lanes_ + q] += (uint64_t)w;
@@ -51,25 +57,27 @@ class ServeQueues {
       if (busiest(l) < busiest(best)) best = l;
     return best;
   }
-  // A kernel stream; a direct request that moves half a MB or more finds
-  // another queue when every lane is busy.  Its kernel spends most of its
-  // time waiting for the host link, so three times as many of them in flight
-  // keep the link busier (200 requests of 2^12 .. 2^14, up to 8 primes, 8
-  // lanes: 1.23 ms on the kernel streams alone, 1.10 with the others).
-  // Smaller ones keep to the lanes: there the server thread's issue time is
-  // the bound, and launches on more streams cost it more (1000 requests of
-  // 2^10 .. 2^12: 4.4 -> 4.7 us each).
+  // A kernel stream; a direct request of a MB or more finds another queue
+  // when every lane is busy.  Its kernel spends most of its time waiting for
+  // the host link, so three times as many of them in flight keep the link
+  // busier (200 requests of 2^12 .. 2^14, up to 8 primes, 8 lanes: 1.23 ms on
+  // the kernel streams alone, 1.07 with the others from 1 MB, 1.10 from 1.4).
+  // The link moves a MB in about the 4.4 us that the server thread needs per
+  // request: below that the thread is the bound, and launches on more streams
+  // cost it more (1000 requests of 2^10 .. 2^12, up to 8 primes: 4.51 ms from
+  // 1 MB, 4.65 from half a MB; 300 of 2^12, 2^13: 1.47 / 1.52).
   int pick_direct(uint64_t weight) const {
     int best = 0;
     for (int l = 1; l < lanes_; ++l)
       if (load_[l] < load_[best]) best = l;
-    if (weight >= (512u << 10) && load_[best] > 0)
+    if (weight >= (1u << 20) && load_[best] > 0)
       for (int l = lanes_; l < queues(); ++l)
         if (load_[l] < load_[best]) best = l;
     return best;
   }
 
   int lanes_ = 0;
+  int beyond_ = 0;              // direct requests on queues past the lanes
   std::vector<uint64_t> load_;  // bytes of the requests in flight on each queue
 };
 

@@ -68,6 +68,31 @@ def test_queue_choice(tmp_path):
     assert r.returncode == 0, r.stdout
 
 
+HOST_SMALL = r"""
+#include "serve_queue.h"
+int main() {
+  pm::ServeQueues s;
+  s.reset(2);
+  // below a MB a direct request stays on a lane, however busy
+  for (int i = 0; i < 8; ++i)
+    if (s.admit(true, 768 << 10) >= 2) return 1;
+  if (s.occupied() != 2) return 2;
+  // the queues past the lanes are looked at only while one holds a request
+  const int q = s.admit(true, 2 << 20);
+  if (q < 2 || s.occupied() != 6) return 3;
+  s.release(q, true, 2 << 20);
+  return s.occupied() != 2;
+}
+"""
+
+
+def test_small_requests_keep_to_the_lanes(tmp_path):
+    src, exe = tmp_path / "small.cpp", tmp_path / "small"
+    src.write_text(HOST_SMALL)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", CSRC, str(src), "-o", str(exe)])
+    assert subprocess.run([str(exe)]).returncode == 0
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("bits", [59, 61])
 def test_mixed_routes(bits):
