@@ -489,11 +489,10 @@ int polymul_ragged_status(polymul_ragged_batch *batch, void *stream);
  * polymul_ragged_tune -- choose the kernel shapes and paths of a prepared
  * list by measurement on the caller's operands (the paper leaves such
  * dimensions to experiment, Sec. 2.6).  Each of the list's two NTT launches
- * (degrees 2^10 .. 2^13; 2^14) exists in two shape sets -- 0: swizzled
- * exchanges, both operands in registers (2^14: the batch kernel, the
- * default there); 1: padded exchanges at half the registers (the default
- * for 2^10 .. 2^13, where lists of up to 13000 coefficients per SM take set
- * 0; 2^14: one operand in registers at a time) -- and each launch keeps the
+ * (degrees 2^10 .. 2^13; 2^14) exists in two shape sets -- 0: 128 registers,
+ * one operand at a time at 2^10, 2^11 (2^14: the batch kernel, the default
+ * there); 1: half the registers, both operands (2^14: one operand at a time);
+ * by default 2^10 .. 2^13 take set 1 for long lists -- and each launch keeps the
  * faster set; then each degree class runs on the path that is
  * faster for its rows: its NTT segment alone, or the tensor path (Sec. 2.2
  * matrix form: the tiled digit kernel with 8-bit digits drained per K

@@ -70,8 +70,8 @@ bool lookup_ntt_cluster2(uint32_t elem, int logn, int mode, bool seq, KernelInfo
 bool lookup_ntt_cluster_small(uint32_t elem, int logn, int mode, KernelInfo* ki);
 
 // uneven batches (32-bit words): one persistent kernel for the degrees
-// 2^10..2^13 and one for 2^14, in two shape sets (0: swizzled exchanges,
-// both operands; 1: padded exchanges, one operand at 2^10, 2^11 and 2^14)
+// 2^10..2^13 and one for 2^14, in two shape sets (see RaggedShape in
+// ragged.cu): 0 for short lists, 1 for long ones
 constexpr int kRaggedSets = 2;
 constexpr int kRaggedClasses = 5;  // degree classes 2^10 .. 2^14 of an uneven list
 bool lookup_ntt_ragged(int mode, int set, KernelInfo* small, KernelInfo* big);

@@ -145,21 +145,36 @@ __device__ __forceinline__ uint32_t xpos(uint32_t j) {
 //          it back below 2q at the pass's end (15 subtractions per 16
 //          coefficients and four stages instead of 32).
 enum { kQ31 = 0, kL4 = 1, kSmall = 2, kTiny = 3, kLazy = 4 };
+// A bit beside the mode, 32-bit words: conditional subtractions as a
+// subtraction and a minimum instead of the fused instruction.  The uneven
+// lists' kernel of 16 warps per SM takes it (4.5 M coefficients of 2^10, 2^11:
+// 44.1 us, fused 45.8; 60 lists of one to four degrees: 0 - 5 % faster so);
+// their kernel of 32 warps gains nothing and loses up to 11 % (2^10 .. 2^14).
+constexpr int kApart = 8;
+constexpr int base_mode(int mode) { return mode & 7; }
+
+template <int MODE, typename W>
+__device__ __forceinline__ W csub_in(W x, W m) {
+  if constexpr ((MODE & kApart) != 0)
+    return csub<W>(x, m);  // the generic form
+  else
+    return csub(x, m);
+}
 
 template <typename W, int MODE>
 __device__ __forceinline__ void ct_bfly(W& x, W& y, const TwPair<W>& w, const PrimeConst<W>& pc) {
-  if constexpr (MODE == kSmall || MODE == kLazy) {
+  if constexpr (base_mode(MODE) == kSmall || MODE == kLazy) {
     W t = shoup(y, w.w, w.wp, pc.q);
     y = x - t + pc.q2;
     x = x + t;
-  } else if constexpr (MODE == kL4) {
-    W xr = csub(x, pc.q2);
+  } else if constexpr (base_mode(MODE) == kL4) {
+    W xr = csub_in<MODE>(x, pc.q2);
     W t = shoup(y, w.w, w.wp, pc.q);
     x = xr + t;
     y = xr - t + pc.q2;
   } else {
-    W xr = csub(x, pc.q);
-    W t = csub(shoup(y, w.w, w.wp, pc.q), pc.q);
+    W xr = csub_in<MODE>(x, pc.q);
+    W t = csub_in<MODE>(shoup(y, w.w, w.wp, pc.q), pc.q);
     x = xr + t;
     y = xr - t + pc.q;
   }
@@ -188,17 +203,17 @@ __device__ __forceinline__ W lazy_reduce(W x, const PrimeConst<W>& pc) {
 // kLazy: the growth of both slots in this pass)
 template <typename W, int MODE, int H>
 __device__ __forceinline__ void gs_bfly(W& x, W& y, W w, W wp, const PrimeConst<W>& pc) {
-  if constexpr (MODE == kSmall || MODE == kLazy) {
+  if constexpr (base_mode(MODE) == kSmall || MODE == kLazy) {
     W d = x - y + (pc.q << (H + 1));
     x = x + y;
     y = shoup(d, w, wp, pc.q);
-  } else if constexpr (MODE == kL4) {
+  } else if constexpr (base_mode(MODE) == kL4) {
     W s = x + y;
     W d = x - y + pc.q2;
-    x = csub(s, pc.q2);
+    x = csub_in<MODE>(s, pc.q2);
     y = shoup(d, w, wp, pc.q);
   } else {
-    W xr = csub(x, pc.q), yr = csub(y, pc.q);
+    W xr = csub_in<MODE>(x, pc.q), yr = csub_in<MODE>(y, pc.q);
     W d = xr - yr + pc.q;
     x = xr + yr;
     y = shoup(d, w, wp, pc.q);
@@ -209,14 +224,14 @@ __device__ __forceinline__ void gs_bfly(W& x, W& y, W w, W wp, const PrimeConst<
 template <typename W, int MODE, int H>
 __device__ __forceinline__ void gs_last(W& x, W& y, const PrimeConst<W>& pc) {
   W s, d;
-  if constexpr (MODE == kSmall || MODE == kLazy) {
+  if constexpr (base_mode(MODE) == kSmall || MODE == kLazy) {
     s = x + y;
     d = x - y + (pc.q << (H + 1));
-  } else if constexpr (MODE == kL4) {
+  } else if constexpr (base_mode(MODE) == kL4) {
     s = x + y;
     d = x - y + pc.q2;
   } else {
-    W xr = csub(x, pc.q), yr = csub(y, pc.q);
+    W xr = csub_in<MODE>(x, pc.q), yr = csub_in<MODE>(y, pc.q);
     s = xr + yr;
     d = xr - yr + pc.q;
   }
@@ -571,21 +586,21 @@ __device__ __forceinline__ void polymul_unit(W* __restrict__ c, const TwPair<W>*
   // pointwise product in the bit-reversed domain (same layout for both)
   sfor<0, S::R>([&](auto ec) {
     constexpr int e = decltype(ec)::value;
-    if constexpr (MODE == kSmall) {
+    if constexpr (base_mode(MODE) == kSmall) {
       xa[e] = montmul(xa[e], xb[e], pc.q, pc.qinv);
     } else if constexpr (MODE == kLazy) {
       xa[e] = lazy_product(xa[e], xb[e], pc);
-    } else if constexpr (MODE == kL4) {
-      xa[e] = csub(montmul(xa[e], xb[e], pc.q, pc.qinv), pc.q2);
+    } else if constexpr (base_mode(MODE) == kL4) {
+      xa[e] = csub_in<MODE>(montmul(xa[e], xb[e], pc.q, pc.qinv), pc.q2);
     } else {
-      xa[e] = montmul(csub(xa[e], pc.q), csub(xb[e], pc.q), pc.q, pc.qinv);
+      xa[e] = montmul(csub_in<MODE>(xa[e], pc.q), csub_in<MODE>(xb[e], pc.q), pc.q, pc.qinv);
     }
   });
   inv_from<S, MODE, 0>(xa, sa, twi, pc, t, sync, hook);
   if (act) {
     sfor<0, S::R>([&](auto ec) {
       constexpr int e = decltype(ec)::value;
-      W y = csub(xa[e], pc.q);
+      W y = csub_in<MODE>(xa[e], pc.q);
       if constexpr (AUX) {
         // centre mod p, then reduce mod qo
         if (y > (pc.q >> 1)) {
@@ -635,14 +650,14 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
   sfor<0, S::R>([&](auto ec) {
     constexpr int e = decltype(ec)::value;
     const W y = sa[e * S::T + t];
-    if constexpr (MODE == kSmall) {
+    if constexpr (base_mode(MODE) == kSmall) {
       x[e] = montmul(y, x[e], pc.q, pc.qinv);
     } else if constexpr (MODE == kLazy) {
       x[e] = lazy_product(y, x[e], pc);
-    } else if constexpr (MODE == kL4) {
-      x[e] = csub(montmul(y, x[e], pc.q, pc.qinv), pc.q2);
+    } else if constexpr (base_mode(MODE) == kL4) {
+      x[e] = csub_in<MODE>(montmul(y, x[e], pc.q, pc.qinv), pc.q2);
     } else {
-      x[e] = montmul(csub(y, pc.q), csub(x[e], pc.q), pc.q, pc.qinv);
+      x[e] = montmul(csub_in<MODE>(y, pc.q), csub_in<MODE>(x[e], pc.q), pc.q, pc.qinv);
     }
   });
   if constexpr (S::NPH == 1) {
@@ -653,7 +668,7 @@ __device__ __forceinline__ void polymul_unit_seq(W* __restrict__ c, const TwPair
   if (act) {
     sfor<0, S::R>([&](auto ec) {
       constexpr int e = decltype(ec)::value;
-      W y = csub(x[e], pc.q);
+      W y = csub_in<MODE>(x[e], pc.q);
       if constexpr (AUX) {
         if (y > (pc.q >> 1)) {
           const W r = (pc.q - y) % qo;

@@ -36,20 +36,23 @@ struct TeamSync {
 
 // degree class -> register radix (16 coefficients per thread up to 2^13,
 // 32 for 2^14 so that a unit fits in 512 threads).  Two shape sets, chosen
-// per list by measurement (polymul_ragged_tune):
-//   set 0: the XOR-swizzled exchange layout, both operands in registers;
-//   set 1: the padded layout (one word after every 2^RB, a base register
-//          plus constant offsets per layout); 2^10 .. 2^13 at 64 registers,
-//          two CTAs and 32 warps per SM (the multiply pipe is the bound, and
-//          16 warps left it idle at barriers and exchanges: the 2000-product
-//          list 1.045 -> 0.895 ms with this set and the batch kernel for
-//          2^14); 2^14 one operand in registers at a time.
+// per list by its sizes (polymul_ragged_prepare) or by measurement
+// (polymul_ragged_tune):
+//   set 0: 2^10 .. 2^13 padded (one word after every 2^RB, a base register
+//          plus constant offsets per layout), 128 registers, one CTA of 16
+//          warps per SM, one operand in registers at a time for 2^10, 2^11:
+//          short lists, where a unit's latency decides;
+//   set 1: the same layout at 64 registers, both operands, two CTAs and 32
+//          warps per SM (the multiply pipe is the bound, and 16 warps left it
+//          idle at barriers and exchanges: the 2000-product list 955 -> 895
+//          us); 2^14 padded, one operand at a time (set 0 of 2^14 is the batch
+//          kernel, see ragged_api.cu).
 constexpr int ragged_rb(int logn) { return logn <= 13 ? 4 : 5; }
 template <int LOGN, int SET>
-using RaggedShape = Shape<uint32_t, LOGN, ragged_rb(LOGN), SET == 1 ? ragged_rb(LOGN) : 0>;
+using RaggedShape = Shape<uint32_t, LOGN, ragged_rb(LOGN), (LOGN <= 13 || SET == 1) ? ragged_rb(LOGN) : 0>;
 template <int LOGN, int SET>
 constexpr bool ragged_seq() {
-  return SET == 1 && LOGN == 14;
+  return SET == 0 ? LOGN == 10 || LOGN == 11 : LOGN == 14;
 }
 
 // One degree segment: the units of degree 2^LOGN, taken one at a time by
@@ -144,8 +147,8 @@ __global__ void __launch_bounds__(kRaggedThreads, (SET == 1 && HI <= 13) ? 2 : 1
 #define PM_SEG(L)                                                                                      \
   case L:                                                                                              \
     if constexpr (L >= LO && L <= HI) {                                                                 \
-      ok = ragged_segment<RaggedShape<L, SET>, MODE, ragged_seq<L, SET>()>(args, seg, ctr, smem, mbar,  \
-                                                                           phases, s_next, bits);       \
+      ok = ragged_segment<RaggedShape<L, SET>, SET == 0 ? MODE | kApart : MODE, ragged_seq<L, SET>()>(   \
+          args, seg, ctr, smem, mbar, phases, s_next, bits);                                            \
       teams = kRaggedThreads / RaggedShape<L, SET>::T;                                                  \
     }                                                                                                   \
     break;

@@ -69,8 +69,8 @@ struct polymul_ragged_batch {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   cudaGraphNode_t node[2] = {nullptr, nullptr};
-  // shape set of each launch: the padded set for 2^10 .. 2^13 (short lists:
-  // set 0, see polymul_ragged_prepare), the batch kernel for 2^14 by default;
+  // shape set of each launch: by the list's sizes for 2^10 .. 2^13 (see
+  // polymul_ragged_prepare), the batch kernel for 2^14 by default;
   // polymul_ragged_tune measures both
   int set[2] = {1, 0};
   // degree segments of the whole list (host copy; d_items holds those the
@@ -381,15 +381,27 @@ extern "C" int polymul_ragged_prepare(polymul_ragged* r, const polymul_desc* des
   }
   b->items_h = items;
   for (const RaggedItem& it : items) b->present |= 1u << (it.logn - 10);
-  // Short lists take set 0 for the smaller degrees: with one or two units per
-  // team a unit's latency decides, and the 64-register body of set 1 is the
-  // longer one (483 rows of 2^10: 14.7 us against 20.0; 287 rows of 2^11 ..
-  // 2^14 30.3 / 33.2; 448 rows of 2^12, 2^13, 2.7 M coefficients, 39.3 / 38.2;
-  // 3119 rows, 15 M coefficients, 174 / 142).
-  uint64_t small_coeffs = 0;
-  for (const RaggedItem& it : items)
-    if (it.logn < 14) small_coeffs += (uint64_t)it.count << it.logn;
-  if (small_coeffs <= 13000ull * (uint64_t)r->num_sms) b->set[0] = 0;
+  // The smaller degrees' set.  With a few units per team a unit's latency
+  // decides, and set 1's is longer (600 rows of 2^10: 14.6 us, set 1 21.7; 600
+  // of 2^11 16.0 / 24.9); what set 1 gains is throughput, and most of it where
+  // teams are large: barriers of 512 threads at 2^13, and the wait between
+  // segments.  Lists with a quarter of their coefficients at 2^13: the two
+  // meet at 19000 coefficients per SM (10^3 per SM, set 0 / 1: 2^12, 2^13 18
+  // 38.7 / 39.0 us, 24 44.6 / 42.6, 37 81.3 / 65.4; 2^10 .. 2^13 15 31.0 / 33.1,
+  // 23 44.6 / 43.7, 33 67.8 / 63.4).  Others of three degrees: at 40000 (33
+  // 53.4 / 56.2, 42 60.5 / 59.7, 47 69.9 / 66.2).  One or two degrees: within
+  // 3 % of each other from 50000 on, set 1 ahead from 100000 (2^11, 2^12: 42
+  // 61.9 / 63.8, 61 81.5 / 84.5, 118 141.7 / 139.0, 250 278 / 272).
+  uint64_t coeffs = 0, coeffs13 = 0;
+  int degrees = 0;
+  for (const RaggedItem& it : items) {
+    if (it.logn >= 14) continue;
+    coeffs += (uint64_t)it.count << it.logn;
+    if (it.logn == 13) coeffs13 = (uint64_t)it.count << 13;
+    ++degrees;
+  }
+  const uint64_t line = 4 * coeffs13 >= coeffs ? 19000 : degrees >= 3 ? 40000 : 100000;
+  if (coeffs <= line * (uint64_t)r->num_sms) b->set[0] = 0;
   apply_paths(b);
   *out = b;
   return POLYMUL_OK;
