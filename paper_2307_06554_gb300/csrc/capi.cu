@@ -309,7 +309,8 @@ int upload_tensor_tables(polymul_plan* p) {
 // for its moduli too.
 int cluster_mode(uint32_t elem, int mode) { return mode != 2 ? mode : elem == 8 ? 4 : 1; }
 
-bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
+// the default kernel; `overlap`: for a plan with POLYMUL_FLAG_OVERLAP
+bool lookup_ntt(uint32_t elem, int logn, int mode, bool overlap, KernelInfo* ki) {
   // n = 2^14, 32-bit words: one 512-thread CTA per product (32 coefficients
   // per thread) beats the two-CTA cluster (measured 101.9 vs 160.8 us for
   // 512 products); the cluster kernel stays an autotuner candidate
@@ -324,7 +325,7 @@ bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
   }
   if (elem == 4) {
     if (mode == 0) return lookup_ntt_u32_m0(logn, ki);
-    if (mode == 1) return lookup_ntt_u32_m1(logn, ki);
+    if (mode == 1) return (overlap && lookup_ntt_u32_m1_seq(logn, ki)) || lookup_ntt_u32_m1(logn, ki);
     return lookup_ntt_u32_m2(logn, ki);
   }
   if (mode == 1) return lookup_ntt_u64_m1(logn, ki);
@@ -450,7 +451,8 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   }
   p->mode = ntt_mode(qmax, p->logn, p->elem);
   if (p->mode < 0) ntt_ok = false;
-  if (ntt_ok && !lookup_ntt(p->elem, (int)p->logn, p->mode, &p->ki)) ntt_ok = false;
+  const bool overlap = (p->flags & POLYMUL_FLAG_OVERLAP) != 0;
+  if (ntt_ok && !lookup_ntt(p->elem, (int)p->logn, p->mode, overlap, &p->ki)) ntt_ok = false;
 
   // auxiliary-prime NTT: one 31-bit prime carries the exact integer product
   bool aux_ok = false;

@@ -31,6 +31,7 @@ struct KernelInfo {
 // 1 = kL4, 2 = kSmall, 4 = kLazy; see ntt.cuh)
 bool lookup_ntt_u32_m0(int logn, KernelInfo* ki);  // logn 4..14
 bool lookup_ntt_u32_m1(int logn, KernelInfo* ki);
+bool lookup_ntt_u32_m1_seq(int logn, KernelInfo* ki);  // one operand at a time: logn 10, 11
 bool lookup_ntt_u32_m2(int logn, KernelInfo* ki);
 bool lookup_ntt_u64_m1(int logn, KernelInfo* ki);  // logn 4..13
 bool lookup_ntt_u64_m2(int logn, KernelInfo* ki);

@@ -13,13 +13,17 @@ constexpr int kNttWarps = 4;  // warps per CTA when a team fits in a warp
 // and whether one operand at a time is held in registers (SEQ).  Measured on
 // GB300 with 2^22 coefficients per batch (2^21 for 64-bit words), launches
 // back to back:
-//   32-bit words, n <= 2^11:     radix 16, padded, 96 registers, both operands
-//                                 (one operand at a time at 2^10, 2^11: 29.7
-//                                 and 32.5 us against 28.5 and 30.3 for 4 M
-//                                 coefficients, q < 2^30; 64 registers win only
-//                                 beyond 16 M), except
-//   ... unreduced mode, 2^10, 2^11: one operand (n = 1024, q = 12289: 27.0 ->
-//                                 25.7 us);
+//   32-bit words, n <= 2^9:      radix 16, padded, 96 registers, both operands;
+//   32-bit words, 2^10, 2^11:    radix 16, padded, 96 registers, one operand
+//                                 (n = 1024, q = 12289: 27.0 -> 25.7 us; 31-bit
+//                                 primes, 3 M coefficients: 22.5 us at 2^10,
+//                                 both operands 23.6; 24.0 / 25.1 at 2^11),
+//                                 except
+//   ... Harvey's bounds:         both operands, without POLYMUL_FLAG_OVERLAP
+//                                 (q < 2^30, 3.2 M coefficients, one operand /
+//                                 both: 23.6 / 22.7 us at 2^10, 24.4 / 24.3 at
+//                                 2^11; overlapped 19.3 / 19.9 and 20.2 / 21.3:
+//                                 see lookup_ntt_u32_m1_seq);
 //   32-bit words, n >= 2^12:     radix 16, padded, 64 registers, both operands:
 //                                 32 warps per SM hold the multiply pipe at
 //                                 74 % of its cycles.  16 M coefficients,
@@ -46,7 +50,7 @@ template <typename W, int LOGN, int MODE = 1>
 struct NttCfg {
   static constexpr bool u32 = sizeof(W) == 4;
   static constexpr int RB = u32 ? 4 : (LOGN >= 6 && LOGN <= 12 ? 3 : 4);
-  static constexpr bool SEQ = u32 ? MODE == kSmall && (LOGN == 10 || LOGN == 11) : (LOGN >= 6 && LOGN <= 11);
+  static constexpr bool SEQ = u32 ? MODE != kL4 && (LOGN == 10 || LOGN == 11) : (LOGN >= 6 && LOGN <= 11);
   static constexpr int PAD = u32 ? (LOGN >= 5 ? 4 : 0) : (LOGN >= 6 ? RB : 0);
   static constexpr int REGS = u32 ? (LOGN < 5 ? 128 : LOGN < 12 ? 96 : 64) : (LOGN >= 6 && LOGN <= 11 ? 96 : LOGN == 12 ? 64 : 128);
 };
@@ -58,7 +62,7 @@ KernelInfo ntt_info_x() {
   KernelInfo ki;
   ki.fn = (const void*)k_ntt_batch<S, MODE, kNttWarps, REGS, AUX, SEQ, DIRECT>;
   ki.rb = RB;
-  ki.mode = MODE;
+  ki.mode = base_mode(MODE);
   ki.regs = REGS;
   ki.pad = PAD;
   ki.seq = SEQ ? 1 : 0;

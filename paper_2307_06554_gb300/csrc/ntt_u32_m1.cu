@@ -15,4 +15,12 @@ bool lookup_ntt_u32_m1(int logn, KernelInfo* ki) {
       return false;
   }
 }
+
+// One operand in registers at a time, for overlapped batches at 2^10, 2^11:
+// the faster shape there (see NttCfg), as the other modes' default is.
+bool lookup_ntt_u32_m1_seq(int logn, KernelInfo* ki) {
+  if (logn == 10) *ki = ntt_info_x<uint32_t, 10, 1, false, 4, 96, 4, true>();
+  if (logn == 11) *ki = ntt_info_x<uint32_t, 11, 1, false, 4, 96, 4, true>();
+  return logn == 10 || logn == 11;
+}
 }  // namespace pm
