@@ -484,7 +484,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   };
 
   int rc = POLYMUL_OK;
-  size_t few = 0;  // the candidate for few products, if there is one
+  size_t few = 0;  // the candidate for few products (2^12, 2^13: other sizes), if there is one
   // NTT batch kernels take a programmatic dependent launch (measured on
   // back-to-back batches: n = 1024, 4096 products 29.9 -> 27.6 us; n = 256,
   // 64 products 8.3 -> 5.7 us); cluster and tensor kernels take plain launches
@@ -548,10 +548,8 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     }
     if (rc == POLYMUL_OK && p->logn < 14 && lookup_ntt_alt(p->elem, (int)p->logn, p->mode, &v)) {
       rc = add_candidate(POLYMUL_PATH_NTT, v);
-      // 32-bit words, n = 2^13, one product per SM at most: nothing else runs
-      // beside it, and 128 registers hold more loads in flight (125 products,
-      // q < 2^20: 12.7 us against 13.3)
-      if (p->elem == 4 && p->logn == 13) few = p->cands.size() - 1;
+      // 32-bit words, n = 2^12, 2^13: for some batch sizes, see below
+      if (p->elem == 4 && p->logn >= 12) few = p->cands.size() - 1;
     }
     // n >= 2^13 (64-bit words), 2^14 (32-bit): few products over more CTAs
     // each, up to the number at which that no longer pays.  64-bit words: at
@@ -568,12 +566,33 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   }
   if (rc == POLYMUL_OK) apply_candidate(p, 0);
   if (rc == POLYMUL_OK && few) {
-    p->small = few;
+    p->other.cand = few;
     const uint64_t sms = (uint64_t)p->num_sms;
-    if (p->elem == 8)
-      p->small_line = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
-    else
-      p->small_line = p->logn == 14 ? sms / 2 : p->logn == 13 ? sms : sms * 2048 / p->n;
+    if (p->elem == 8) {
+      p->other.upto = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
+    } else if (p->logn == 14) {
+      p->other.upto = sms / 2;
+    } else if (p->logn >= 12) {
+      // The 128-register kernel beside the 64-register default.  2^13, one
+      // product per SM at most: nothing else runs beside it, and 128 registers
+      // hold more loads in flight (125 products, q < 2^20: 12.7 us against
+      // 13.3).  Overlapped batches: the next one's CTAs start as this one's
+      // leave, and with fewer resident CTAs, each taking several products, they
+      // fill the SMs evenly, where the default runs in whole waves of two CTAs
+      // per SM at 2^13, four at 2^12 (2^13, q < 2^30, default / this, batches
+      // of 156 20.4 / 15.9 us, 230 20.7 / 17.7, 304 20.8 / 21.7, 320 29.1 /
+      // 23.0, 410 32.0 / 29.4, 480 35.9 / 34.2, 520 35.5 / 36.8; 2^12, 500
+      // 17.1 / 15.3, 830 26.5 / 23.7, 1216 36.5 / 33.5, 1600 43.6 / 44.1).
+      const bool overlap = (p->flags & POLYMUL_FLAG_OVERLAP) != 0;
+      if (p->logn == 13) {
+        p->other.upto = overlap ? 15 * sms / 8 : sms;
+        if (overlap) p->other.lo = 2 * sms, p->other.hi = 13 * sms / 4;
+      } else if (overlap) {
+        p->other.upto = 9 * sms;
+      }
+    } else {
+      p->other.upto = sms * 2048 / p->n;
+    }
   }
   // Small batches leave most of the GPU idle whatever the kernel: one unit's
   // latency is the call, and more threads per unit with shorter chains win.
@@ -586,11 +605,11 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   if (rc == POLYMUL_OK && p->cands.size() > 1) {
     const bool aux2 = p->aux_prime != 0;
     if (aux2 || p->cands[0].ki.tiny) {
-      p->small = 1;
-      p->small_line = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
+      p->other.cand = 1;
+      p->other.upto = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
     }
   }
-  p->small_units = p->small_line;
+  p->other_on = p->other.upto > 0;
   if (rc == POLYMUL_OK) {
     // work counters for the three launch slots (device entry, two host-entry streams)
     if (cudaMalloc(&p->d_ctr, 2 * kCounterSlots * sizeof(unsigned long long)) != cudaSuccess ||
@@ -800,13 +819,13 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     const int r = validate_operands(p, a, b, units, st);
     if (r != POLYMUL_OK) return r;
   }
-  // the kernel: the plan's choice, or the candidate for batches this small
+  // the kernel: the plan's choice, or the candidate for batches of this size
   // (a pending diagnostics injection counts launches of the batch kernel, so
   // it keeps the plan's choice)
-  const PlanCandidate* small =
-      units <= p->small_units && !injected_wait_pending() ? &p->cands[p->small] : nullptr;
-  const KernelInfo& ki = small ? small->ki : p->ki;
-  const int grid_cap = small ? small->grid_cap : p->grid_cap;
+  const PlanCandidate* other =
+      p->other_on && p->other.takes(units) && !injected_wait_pending() ? &p->cands[p->other.cand] : nullptr;
+  const KernelInfo& ki = other ? other->ki : p->ki;
+  const int grid_cap = other ? other->grid_cap : p->grid_cap;
   const uint64_t need = (units + ki.units_per_cta - 1) / ki.units_per_cta;
   int grid = (int)std::min<uint64_t>(need, (uint64_t)grid_cap);
   int smem = ki.smem;

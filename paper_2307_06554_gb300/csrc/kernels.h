@@ -43,8 +43,9 @@ bool lookup_ntt_u32_aux_rb2(int logn, KernelInfo* ki);  // the same with radix-4
 bool lookup_ntt_u32_rb5(int logn, int mode, KernelInfo* ki);  // logn 9..13, modes 1, 2; logn 14, modes 0..2
 bool lookup_ntt_u32_rb3(int logn, int mode, KernelInfo* ki);  // logn 9..12, modes 1, 2
 // the alternative shape of the default kernel's measurements (the other
-// layout / operand scheme): 32-bit words, modes 1, 2, logn 5..13; 64-bit
-// words, mode 1, logn 6..12
+// layout / operand scheme): 32-bit words, mode 0, logn 12, 13, modes 1, 2,
+// logn 5..13; 64-bit words, modes 1, 4 (both the Harvey-bound kernels), logn
+// 6..12
 bool lookup_ntt_alt(uint32_t elem, int logn, int mode, KernelInfo* ki);
 
 // the batch kernel reading a and b and writing c where they lie (host

@@ -5,11 +5,13 @@
 
 namespace pm {
 
+bool lookup_ntt_alt_u32_m0(int logn, KernelInfo* ki);
 bool lookup_ntt_alt_u32_m1(int logn, KernelInfo* ki);
 bool lookup_ntt_alt_u32_m2(int logn, KernelInfo* ki);
 
 bool lookup_ntt_alt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
   if (elem == 4) {
+    if (mode == 0) return lookup_ntt_alt_u32_m0(logn, ki);
     if (mode == 1) return lookup_ntt_alt_u32_m1(logn, ki);
     if (mode == 2) return lookup_ntt_alt_u32_m2(logn, ki);
     return false;

@@ -23,6 +23,14 @@ struct PlanCandidate {
 
 constexpr uint32_t kLaunchPdl = 2u;  // programmatic dependent launch
 
+// A candidate that batches of certain sizes take instead of the default one:
+// those of at most `upto` units, and those of more than `lo` and at most `hi`.
+struct BatchRule {
+  size_t cand = 0;
+  uint64_t upto = 0, lo = 0, hi = 0;
+  bool takes(uint64_t units) const { return units <= upto || (units > lo && units <= hi); }
+};
+
 struct polymul_plan {
   uint32_t n = 0, logn = 0, k = 0;
   uint32_t elem = 4;   // bytes per coefficient word (4 or 8)
@@ -48,12 +56,11 @@ struct polymul_plan {
   pm::KernelInfo tki;  // tensor-path kernel, when one exists for the shape
   std::vector<PlanCandidate> cands;  // [0] is the default
   size_t chosen = 0;
-  // batches of at most small_units units run candidate `small` instead of
-  // the default one (see polymul_create); 0: none.  small_line is that limit
-  // as created: small_units is 0 while another candidate, or explicitly the
-  // default one (polymul_plan_select), is chosen
-  size_t small = 0;
-  uint64_t small_units = 0, small_line = 0;
+  // batches that run another candidate than the default one (see
+  // polymul_create); `other_on`: the rule holds, i.e. the choice is the
+  // default one and not an explicit one (polymul_plan_select)
+  BatchRule other;
+  bool other_on = false;
   bool tuned = false;
   uint64_t tuned_batch = 0;  // batch bucket of the tuned choice
   void* d_tpc = nullptr;  // tensor-path constants
@@ -99,7 +106,7 @@ struct polymul_plan {
 
 inline void apply_candidate(polymul_plan* p, size_t i) {
   p->chosen = i;
-  p->small_units = 0;
+  p->other_on = false;
   p->path = p->cands[i].path;
   p->ki = p->cands[i].ki;
   p->grid_cap = p->cands[i].grid_cap;

@@ -77,11 +77,11 @@ std::string label_of(const PlanCandidate& c) {
   return buf;
 }
 
-// The tuned choice.  The default candidate keeps its form for small batches,
-// unless it was measured at such a batch and won there.
+// The tuned choice.  The default candidate keeps the kernel that other batch
+// sizes take, unless it was measured at such a size and won there.
 void settle(polymul_plan* p, size_t i, uint64_t bucket) {
   apply_candidate(p, i);
-  if (i == 0 && bucket * p->k > p->small_line) p->small_units = p->small_line;
+  p->other_on = i == 0 && !p->other.takes(bucket * p->k);
   p->tuned = true;
   p->tuned_batch = bucket;
 }
@@ -145,7 +145,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
       cudaEventCreate(&e1) != cudaSuccess)
     rc = fail(POLYMUL_ECUDA, "tuning setup failed");
   const size_t saved_chosen = p->chosen;
-  const uint64_t saved_small = p->small_units;
+  const bool saved_other = p->other_on;
   const uint32_t saved_flags = p->flags;
   p->flags &= ~POLYMUL_FLAG_VALIDATE;
   std::vector<float> best_ms(p->cands.size(), 1e30f);
@@ -196,7 +196,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
   cudaFree(buf);
   if (rc != POLYMUL_OK) {
     apply_candidate(p, saved_chosen);
-    p->small_units = saved_small;
+    p->other_on = saved_other;
     return rc;
   }
   settle(p, best, bucket);
