@@ -583,12 +583,16 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
       // of 156 20.4 / 15.9 us, 230 20.7 / 17.7, 304 20.8 / 21.7, 320 29.1 /
       // 23.0, 410 32.0 / 29.4, 480 35.9 / 34.2, 520 35.5 / 36.8; 2^12, 500
       // 17.1 / 15.3, 830 26.5 / 23.7, 1216 36.5 / 33.5, 1600 43.6 / 44.1).
-      const bool overlap = (p->flags & POLYMUL_FLAG_OVERLAP) != 0;
       if (p->logn == 13) {
         p->other.upto = overlap ? 15 * sms / 8 : sms;
         if (overlap) p->other.lo = 2 * sms, p->other.hi = 13 * sms / 4;
       } else if (overlap) {
         p->other.upto = 9 * sms;
+      } else if (p->mode == 2) {
+        // the unreduced mode multiplies less, and latency weighs more (q < 2^17,
+        // 2^12, default / this: 20 products 8.0 / 7.6 us, 360 15.2 / 14.6, 450
+        // 15.4 / 15.3, 500 18.8 / 19.6)
+        p->other.upto = 3 * sms;
       }
     } else {
       p->other.upto = sms * 2048 / p->n;
@@ -600,14 +604,17 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   // against 6.8; 1024: 5.1 / 8.1) up to 3500 coefficients per SM, where the
   // two meet (n = 512, 1216 units: 8.9 / 8.4).  Smallest moduli: the radix-16
   // kernel (n = 1024, 64 units: 5.4 us against 6.9; n = 256, 152 units:
-  // 5.0 / 6.5) up to 4500 per SM (n = 1024, 608 units 7.5 / 7.5, 912 units
-  // 12.1 / 7.7; n = 256, 2432 units 6.3 / 7.5, 4864 units 9.7 / 7.6).
-  if (rc == POLYMUL_OK && p->cands.size() > 1) {
-    const bool aux2 = p->aux_prime != 0;
-    if (aux2 || p->cands[0].ki.tiny) {
-      p->other.cand = 1;
-      p->other.upto = (uint64_t)p->num_sms * (aux2 ? 3500 : 4500) / p->n;
-    }
+  // 5.0 / 6.5) up to 4800 per SM, 4600 at n = 1024 (n = 256, 2850 units 7.4 /
+  // 8.4, 3265 9.6 / 8.4; n = 1024, 682 units 8.3 / 8.8, 712 8.3 / 8.0), in
+  // overlapped batches up to 4500 (n = 256, 2731 units 5.6 / 5.2), and at n =
+  // 256 where the tiny unit's second CTA on some SMs does not pay yet (32 units
+  // per CTA; 5343 units 9.9 / 10.2, 6234 10.5 / 10.3).
+  if (rc == POLYMUL_OK && p->cands.size() > 1 && (p->aux_prime || p->cands[0].ki.tiny)) {
+    const uint64_t sms = (uint64_t)p->num_sms;
+    const uint64_t per_sm = p->aux_prime ? 3500 : overlap ? 4500 : p->n == 1024 ? 4600 : 4800;
+    p->other.cand = 1;
+    p->other.upto = sms * per_sm / p->n;
+    if (!p->aux_prime && !overlap && p->n == 256) p->other.lo = 32 * sms, p->other.hi = 39 * sms;
   }
   p->other_on = p->other.upto > 0;
   if (rc == POLYMUL_OK) {

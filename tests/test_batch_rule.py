@@ -15,10 +15,12 @@ pytestmark = pytest.mark.gpu
 # n, q or bits, lines (products per SM) of overlapped and of other plans
 CASES = [
     (256, 3329, (3500 / 256,)),          # auxiliary prime
-    (256, 7681, (4500 / 256,)),          # smallest moduli
-    (1024, 12289, (4500 / 1024,)),
+    (256, 7681, (4500 / 256, 4800 / 256, 32, 39)),  # smallest moduli
+    (512, 12289, (4500 / 512, 4800 / 512)),
+    (1024, 12289, (4500 / 1024, 4600 / 1024)),
     (1024, 30, (2,)),
     (2048, 30, (1,)),
+    (4096, 17, (3, 9)),
     (4096, 31, (9,)),
     (4096, 30, (9,)),
     (8192, 31, (1, 15 / 8, 2, 13 / 4)),
