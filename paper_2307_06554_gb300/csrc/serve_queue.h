@@ -40,6 +40,8 @@ class ServeQueues {
   void release(int q, bool direct, uint64_t weight) { add(q, direct, -(int64_t)weight); }
 
  private:
+  static constexpr uint64_t kLarge = 1u << 20;
+
   void add(int q, bool direct, int64_t w) {
     load_[q] += (uint64_t)w;
     if (q >= lanes_) beyond_ += w < 0 ? -1 : 1;
@@ -58,19 +60,22 @@ class ServeQueues {
     return best;
   }
   // A kernel stream; a direct request of a MB or more finds another queue
-  // when every lane is busy.  Its kernel spends most of its time waiting for
-  // the host link, so three times as many of them in flight keep the link
-  // busier (200 requests of 2^12 .. 2^14, up to 8 primes, 8 lanes: 1.23 ms on
-  // the kernel streams alone, 1.07 with the others from 1 MB, 1.10 from 1.4).
+  // when every lane is busy, one of half a MB when every lane has 2 MB ahead.
+  // Its kernel spends most of its time waiting for the host link, so three
+  // times as many of them in flight keep the link busier (200 requests of 2^12
+  // .. 2^14, up to 8 primes, 8 lanes: 1.23 ms on the kernel streams alone).
   // The link moves a MB in about the 4.4 us that the server thread needs per
-  // request: below that the thread is the bound, and launches on more streams
-  // cost it more (1000 requests of 2^10 .. 2^12, up to 8 primes: 4.51 ms from
-  // 1 MB, 4.65 from half a MB; 300 of 2^12, 2^13: 1.47 / 1.52).
+  // request: below that the thread is the bound, unless a backlog shows that
+  // larger requests hold the link, and launches on more streams cost it more.
+  // The other queues for half a MB always / from 2 MB ahead / never: that list
+  // 1.080 / 1.089 / 1.100 ms, 1000 requests of 2^10 .. 2^12 4.57 / 4.46 / 4.47,
+  // 300 of 2^12 1.475 / 1.424 / 1.393.
   int pick_direct(uint64_t weight) const {
     int best = 0;
     for (int l = 1; l < lanes_; ++l)
       if (load_[l] < load_[best]) best = l;
-    if (weight >= (1u << 20) && load_[best] > 0)
+    const uint64_t ahead = load_[best];
+    if ((weight >= kLarge && ahead > 0) || (weight >= kLarge / 2 && ahead >= 2 * kLarge))
       for (int l = lanes_; l < queues(); ++l)
         if (load_[l] < load_[best]) best = l;
     return best;

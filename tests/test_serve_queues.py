@@ -73,10 +73,15 @@ HOST_SMALL = r"""
 int main() {
   pm::ServeQueues s;
   s.reset(2);
-  // below a MB a direct request stays on a lane, however busy
-  for (int i = 0; i < 8; ++i)
+  // below a MB a direct request stays on a lane while the lanes have less than
+  // 2 MB ahead, below half a MB always
+  for (int i = 0; i < 6; ++i)
     if (s.admit(true, 768 << 10) >= 2) return 1;
+  if (s.admit(true, 256 << 10) >= 2) return 1;
   if (s.occupied() != 2) return 2;
+  const int r = s.admit(true, 768 << 10);
+  if (r < 2) return 4;
+  s.release(r, true, 768 << 10);
   // the queues past the lanes are looked at only while one holds a request
   const int q = s.admit(true, 2 << 20);
   if (q < 2 || s.occupied() != 6) return 3;
