@@ -937,9 +937,7 @@ def other_workloads(dev, stream, peaks, alu_peak_g, samples):
                               "units": r.info["units"], "work_items": r.info["items"], "grid": r.info["grid"],
                               "path": "ntt, two concurrent persistent launches (2^14; 2^10..2^13) replayed as a CUDA graph",
                               "shape_sets": {"2^10..2^13": choice & 1, "2^14": (choice >> 1) & 1,
-                                             "legend": "0 swizzled, both operands (at 2^14 the homogeneous "
-                                                       "one-CTA-per-product kernel over the segment's rows); 1 "
-                                                       "padded, one operand at 2^10, 2^11, 2^14 (polymul_ragged_tune)"},
+                                             "legend": "as for polymul_ragged_tune in include/polymul.h"},
                               "alu_frac": mm / (ms / 1e3) / 1e9 / alu_peak_g,
                               "hbm_frac": 3 * total * 4 / (ms / 1e3) / 1e9 / hbm,
                               "bit_exact_sample": None, "l2": "inputs 1.3 GB (> L2)"}
@@ -1641,8 +1639,57 @@ def run_ours(args, ws, rank, local):
         "tensor_path": tensor,
         "other_workloads": extras,
     }
-    print(json.dumps(out), flush=True)
+    # one short line on stdout, everything measured on stderr
+    print("details: " + json.dumps(out), file=sys.stderr, flush=True)
+    print(json.dumps(summary_line(out)), flush=True)
     plan.close()
+
+
+def _short(x):
+    """Six significant digits for every float inside x."""
+    if isinstance(x, float):
+        return float("%.6g" % x)
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [_short(v) for v in x]
+    return x
+
+
+def summary_line(out):
+    """The result line: every field that a reader of one line needs, in under
+    3000 bytes (a log that keeps the last few thousand keeps all of it).
+    Prose, per-leg rooflines and the other workloads' details stay in `out`."""
+    line = {k: out[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "gpu_launches",
+                                "bit_exact_sample", "clocks")}
+    line["config"] = {k: out["config"][k] for k in ("workload", "path", "overlap", "l2", "parallelism")}
+    e2e, roof = out["e2e"], out["roofline"]
+    line["e2e"] = {"value": e2e["value"], "unit": e2e["unit"], "h2d_bytes_per_step": e2e["h2d_bytes_per_step"],
+                   "d2h_bytes_per_step": e2e["d2h_bytes_per_step"], "api": e2e["api"].split(":")[0],
+                   "host_link_frac": (e2e["roofline"] or {}).get("frac"),
+                   "per_call_sync": e2e["per_call_sync"]["value"], "staged": e2e["staged"]["value"]}
+    line["roofline"] = {k: roof[k] for k in ("bound", "achieved", "peak", "unit", "frac", "traffic")}
+    line["roofline"].update(kernel=roof["kernel"].split(" ")[0], hbm_frac=roof["hbm"]["frac"])
+    cpu = out["cpu_baseline"]
+    line["cpu_baseline"] = cpu and {k: cpu[k] for k in ("value", "unit", "cores", "kind")}
+    tensor = out["tensor_path"]
+    line["tensor_path"] = tensor and {"value": tensor["value"], "unit": tensor["unit"],
+                                      "bf16_frac": tensor["roofline"]["frac"],
+                                      "bit_exact_sample": tensor.get("bit_exact_sample")}
+    others = {}
+    for name, x in (out["other_workloads"] or {}).items():
+        if name == "serve_20k":
+            others[name] = {"requests_per_s": x["requests"] / x["saturated"]["seconds"], "exact": x.get("bit_exact_sample")}
+        elif "products_per_s" in x:
+            others[name] = {"products_per_s": x["products_per_s"], "exact": x.get("bit_exact_sample")}
+        else:
+            others[name] = {"rows": len(x["rows"]), "exact": x.get("bit_exact_sample")}
+    line["other_workloads"] = others or None
+    value = line["value"]
+    line = _short(line)
+    line["value"] = value
+    return line
 
 
 def main():
