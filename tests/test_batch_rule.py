@@ -18,8 +18,11 @@ CASES = [
     (256, 7681, (4500 / 256, 4800 / 256, 32, 39)),  # smallest moduli
     (512, 12289, (4500 / 512, 4800 / 512)),
     (1024, 12289, (4500 / 1024, 4600 / 1024)),
+    (512, 30, (4,)),
     (1024, 30, (2,)),
+    (1024, 31, (2,)),
     (2048, 30, (1,)),
+    (2048, 31, (1,)),
     (4096, 17, (3, 9)),
     (4096, 31, (9,)),
     (4096, 30, (9,)),
