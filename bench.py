@@ -456,6 +456,8 @@ def _case(name, launches):
         return _case_homogeneous(4096, wl.draw_primes(rng, 2, 59, 59, 13), 64, polymul.PATH_TENSOR, launches)
     if name == "n16384":
         return _case_homogeneous(16384, wl.draw_primes(rng, 1, 30, 30, 15), 1024, polymul.PATH_NTT, launches)
+    if name == "ntt_rns4096":
+        return _case_homogeneous(4096, wl.draw_primes(rng, 8, 30, 30, 13), 256, polymul.PATH_NTT, launches)
     if name == "cluster_32768":
         return _case_homogeneous(32768, wl.draw_primes(rng, 1, 30, 30, 16), 256, polymul.PATH_NTT, launches)
     if name == "u64_4096":
@@ -479,6 +481,7 @@ CASES = {
     "tensor_u64_4096": "n = 4096, 2 primes of 59 bits, 64 products on the residue-number-system tensor kernel",
     "tensor_u64_16384": "n = 16384, 2 primes of 59 bits, 8 products on the 64-bit-word digit kernel",
     "n16384": "n = 16384, one 30-bit prime, 1024 products (one CTA per product)",
+    "ntt_rns4096": "n = 4096, 8 primes of 30 bits, 256 products (path a, default kernel)",
     "cluster_32768": "n = 32768, one 30-bit prime, 256 products (thread-block clusters)",
     "u64_4096": "n = 4096, one 59-bit prime, 1024 products (64-bit words)",
     "ragged_300": "the first 300 products of the uneven 2000-product list, one persistent launch",
@@ -551,7 +554,8 @@ def _tensor_digits(n: int, qmax: int):
 # ------------------------------------------------------------------ traffic record
 def _kernel_source_hash() -> str:
     h = hashlib.sha256()
-    for fn in ("ntt.cuh", "arith.cuh", "async.cuh", "ntt_info.cuh", "polymul_types.h"):
+    for fn in ("ntt.cuh", "ntt_tiny.cuh", "ntt_tiny_arith.h", "ntt_tiny.cu", "arith.cuh", "async.cuh", "ntt_info.cuh",
+               "polymul_types.h"):
         with open(os.path.join(ROOT, "paper_2307_06554_gb300", "csrc", fn), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]

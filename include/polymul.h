@@ -238,7 +238,9 @@ int polymul_batch(polymul_plan *plan, const void *a, const void *b, void *c,
  *     q < 2^14);
  *   NTT path: a's transform once per modulus, then one forward and one
  *     inverse transform per product (instead of two forward and one
- *     inverse); needs 32-bit words, 1024 <= n <= 8192, a direct NTT.
+ *     inverse); needs 32-bit words, 1024 <= n <= 8192, a direct NTT.  At
+ *     n = 1024 with every q < 18500 one launch does both, each CTA
+ *     transforming a for itself, and needs no scratch.
  * The cyclic flag is honoured.  The plan keeps scratch (digit planes of b
  * and T(a), or a's transforms), grown (cudaMalloc) when a call needs more.
  * Asynchronous; a call must not overlap another call on the same plan (they

@@ -62,13 +62,16 @@ bool lookup_ntt_shared(int logn, int mode, KernelInfo* prep, KernelInfo* main);
 // the same for the smallest moduli (ntt_tiny.cuh) in one launch, logn 10
 bool lookup_ntt_tiny_shared(int logn, KernelInfo* ki);
 
-// one product per thread-block cluster (n = 2^14 .. 2^16)
+// one product per thread-block cluster (n = 2^14 .. 2^16; 32-bit words modes
+// 0 .. 2, 64-bit words modes 1, 2)
 bool lookup_ntt_cluster(uint32_t elem, int logn, int mode, KernelInfo* ki);
 // its second form: CTA-local exchanges except the top phase's, padded
-// layout; one operand in registers at a time (seq) or both (mode 1 only)
+// layout; one operand in registers at a time (seq) or both.  32-bit words
+// modes 0, 1, 64-bit words modes 1, 4 (see cluster_mode in capi.cu)
 bool lookup_ntt_cluster2(uint32_t elem, int logn, int mode, bool seq, KernelInfo* ki);
-// the second form over more CTAs, for few products: 64-bit words n = 2^12 ..
-// 2^15 (mode 1), 32-bit words n = 2^14 (modes 0, 1)
+// the second form over more CTAs, for few products: 64-bit words n = 2^12
+// (mode 1, for the server's direct route) and 2^13 .. 2^15 (modes 1, 4),
+// 32-bit words n = 2^14 (modes 0, 1)
 bool lookup_ntt_cluster_small(uint32_t elem, int logn, int mode, KernelInfo* ki);
 
 // uneven batches (32-bit words): one persistent kernel for the degrees

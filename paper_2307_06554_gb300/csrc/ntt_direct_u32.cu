@@ -12,8 +12,8 @@ bool lookup_ntt_direct_u32(int logn, KernelInfo* ki) {
   switch (logn) {
 #define PM_CASE(L)                                                                                   \
   case L:                                                                                            \
-    *ki = ntt_info_x<uint32_t, L, 0, false, 4, (L >= 5 && L <= 11 ? 96 : 128), (L >= 5 && L <= 11 ? 4 : 0), \
-                     false, true>();                                                                 \
+    *ki = ntt_info_x<uint32_t, L, 0, false, DirectCfg<uint32_t, L>::RB, DirectCfg<uint32_t, L>::REGS, \
+                     DirectCfg<uint32_t, L>::PAD, false, true>();                                    \
     return true;
     PM_CASE(4) PM_CASE(5) PM_CASE(6) PM_CASE(7) PM_CASE(8) PM_CASE(9) PM_CASE(10)
     PM_CASE(11) PM_CASE(12) PM_CASE(13)

@@ -9,8 +9,8 @@ bool lookup_ntt_direct_u64(int logn, KernelInfo* ki) {
   switch (logn) {
 #define PM_CASE(L)                                                                                   \
   case L:                                                                                            \
-    *ki = ntt_info_x<uint64_t, L, 1, false, (L >= 6 && L <= 11 ? 3 : 4), (L >= 6 && L <= 11 ? 96 : 128),  \
-                     (L < 6 ? 0 : L <= 11 ? 3 : 4), false, true>();                                  \
+    *ki = ntt_info_x<uint64_t, L, 1, false, DirectCfg<uint64_t, L>::RB, DirectCfg<uint64_t, L>::REGS, \
+                     DirectCfg<uint64_t, L>::PAD, false, true>();                                    \
     return true;
     PM_CASE(4) PM_CASE(5) PM_CASE(6) PM_CASE(7) PM_CASE(8) PM_CASE(9) PM_CASE(10)
     PM_CASE(11) PM_CASE(12) PM_CASE(13)

@@ -55,6 +55,20 @@ struct NttCfg {
   static constexpr int REGS = u32 ? (LOGN < 5 ? 128 : LOGN < 12 ? 96 : 64) : (LOGN >= 6 && LOGN <= 11 ? 96 : LOGN == 12 ? 64 : 128);
 };
 
+// Shape of the direct kernels (operands in host memory): one per word size and
+// degree, both operands in registers.  The link bounds them, and what counts is
+// loads in flight, so they did not follow the batch kernels to 64 registers
+// (64-bit words, n = 1024, two primes, 89 products through polymul_batch_host:
+// 38.2 us, radix 8 at 64 registers 40.0).
+template <typename W, int LOGN>
+struct DirectCfg {
+  static constexpr bool u32 = sizeof(W) == 4;
+  static constexpr bool mid = LOGN >= (u32 ? 5 : 6) && LOGN <= 11;
+  static constexpr int RB = !u32 && mid ? 3 : 4;
+  static constexpr int REGS = mid ? 96 : 128;
+  static constexpr int PAD = mid ? RB : !u32 && LOGN > 11 ? RB : 0;
+};
+
 // every parameter explicit
 template <typename W, int LOGN, int MODE, bool AUX, int RB, int REGS, int PAD, bool SEQ, bool DIRECT = false>
 KernelInfo ntt_info_x() {

@@ -3,8 +3,8 @@
 // CTAs of eight warps at 96 registers or a little more, two per SM: the
 // unit's straight-line body is long, and warps of one CTA, started together,
 // share its instruction fetch.  n = 1024, q = 12289, overlapped batches of
-// 4096 / 32768 products: 15.3 / 104 us, against 16.9 / 112 with five
-// four-warp CTAs and 22.8 / 175 for the radix-16 kernel of the unreduced
+// 4096 / 32768 products: 15.2 / 104 us, against 16.9 / 112 with five
+// four-warp CTAs and 20.9 / 175 for the radix-16 kernel of the unreduced
 // mode.
 #include "ntt_info.cuh"
 

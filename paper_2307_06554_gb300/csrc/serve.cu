@@ -19,8 +19,9 @@
 // I/O" (ii)).  A request whose a, b and c lie in page-locked host memory the
 // device maps takes the direct route instead: its kernel loads a and b and
 // stores c in host memory itself over the coherent host link, with no arena
-// memory, copy or copy stream (the batch kernel's direct form below 2^14;
-// the cluster kernels load and store with plain accesses already).  Latency
+// memory or copy, on any of a lane's streams (serve_queue.h): the batch
+// kernel's direct form up to 2^11, cluster kernels, which load and store with
+// plain accesses already, above (the small ones to 2^15).  Latency
 // is taken from submission to the moment the server observes completion.
 #include <cuda_runtime.h>
 
@@ -93,8 +94,9 @@ struct polymul_server {
   void* d_pc = nullptr;  // PrimeConst<uint64_t>[pool][17]
   KernelInfo ki[kServeMaxLog + 1];
   int grid_cap[kServeMaxLog + 1] = {};
-  // the direct route's kernel per degree: the batch kernel's direct form
-  // below 2^14, the cluster kernel (ki) from there
+  // the direct route's kernel per degree: the batch kernel's direct form up to
+  // 2^11, the cluster kernel of few products to 2^15, the cluster kernel (ki)
+  // at 2^16
   KernelInfo dki[kServeMaxLog + 1];
   int dgrid_cap[kServeMaxLog + 1] = {};
   std::atomic<int> staged{0};  // polymul_server_set_route: 1 keeps every request on copies
