@@ -213,8 +213,9 @@ int polymul_create(uint32_t n, const uint64_t *q_list, uint32_t k,
  *   stream   cudaStream_t or NULL.
  * A plan whose kernel has not been tuned or selected may run another of its
  * candidates for a batch too small to fill the GPU, with more threads per
- * product; results are the same, and polymul_plan_info describes the kernel
- * of the larger batches.
+ * product, or for one that may start before its predecessor has finished
+ * (POLYMUL_FLAG_OVERLAP); results are the same, and polymul_plan_info
+ * describes the kernel of the other batches.
  * Asynchronous.  The tensor path's residue-number-system kernel keeps
  * residue planes in plan-owned scratch, allocated (or grown) on the first
  * call with a larger batch: make one such call before capturing the stream

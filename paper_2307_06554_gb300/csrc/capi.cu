@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <optional>
 #include <string>
 #include <vector>
 
@@ -309,8 +310,7 @@ int upload_tensor_tables(polymul_plan* p) {
 // for its moduli too.
 int cluster_mode(uint32_t elem, int mode) { return mode != 2 ? mode : elem == 8 ? 4 : 1; }
 
-// the default kernel; `overlap`: for a plan with POLYMUL_FLAG_OVERLAP
-bool lookup_ntt(uint32_t elem, int logn, int mode, bool overlap, KernelInfo* ki) {
+bool lookup_ntt(uint32_t elem, int logn, int mode, KernelInfo* ki) {
   // n = 2^14, 32-bit words: one 512-thread CTA per product (32 coefficients
   // per thread) beats the two-CTA cluster (measured 101.9 vs 160.8 us for
   // 512 products); the cluster kernel stays an autotuner candidate
@@ -325,7 +325,7 @@ bool lookup_ntt(uint32_t elem, int logn, int mode, bool overlap, KernelInfo* ki)
   }
   if (elem == 4) {
     if (mode == 0) return lookup_ntt_u32_m0(logn, ki);
-    if (mode == 1) return (overlap && lookup_ntt_u32_m1_seq(logn, ki)) || lookup_ntt_u32_m1(logn, ki);
+    if (mode == 1) return lookup_ntt_u32_m1(logn, ki);
     return lookup_ntt_u32_m2(logn, ki);
   }
   if (mode == 1) return lookup_ntt_u64_m1(logn, ki);
@@ -452,7 +452,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   p->mode = ntt_mode(qmax, p->logn, p->elem);
   if (p->mode < 0) ntt_ok = false;
   const bool overlap = (p->flags & POLYMUL_FLAG_OVERLAP) != 0;
-  if (ntt_ok && !lookup_ntt(p->elem, (int)p->logn, p->mode, overlap, &p->ki)) ntt_ok = false;
+  if (ntt_ok && !lookup_ntt(p->elem, (int)p->logn, p->mode, &p->ki)) ntt_ok = false;
 
   // auxiliary-prime NTT: one 31-bit prime carries the exact integer product
   bool aux_ok = false;
@@ -485,6 +485,7 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
 
   int rc = POLYMUL_OK;
   size_t few = 0;  // the candidate for few products (2^12, 2^13: other sizes), if there is one
+  size_t one_operand = 0;  // 2^10, 2^11 with Harvey's bounds and POLYMUL_FLAG_OVERLAP: see NttCfg
   // NTT batch kernels take a programmatic dependent launch (measured on
   // back-to-back batches: n = 1024, 4096 products 29.9 -> 27.6 us; n = 256,
   // 64 products 8.3 -> 5.7 us); cluster and tensor kernels take plain launches
@@ -522,6 +523,10 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
     const KernelInfo word = p->ki;
     if (rc == POLYMUL_OK && tiny) rc = add_candidate(POLYMUL_PATH_NTT, v);
     if (rc == POLYMUL_OK) rc = add_candidate(POLYMUL_PATH_NTT, word);
+    if (rc == POLYMUL_OK && overlap && p->elem == 4 && p->mode == 1 && lookup_ntt_u32_m1_seq((int)p->logn, &v)) {
+      rc = add_candidate(POLYMUL_PATH_NTT, v);
+      one_operand = p->cands.size() - 1;
+    }
     if (rc == POLYMUL_OK && p->elem == 4 && lookup_ntt_u32_rb5((int)p->logn, p->mode, &v) && v.fn != p->cands[0].ki.fn)
       rc = add_candidate(POLYMUL_PATH_NTT, v);
     if (rc == POLYMUL_OK && p->elem == 4 && p->logn == 14 &&
@@ -566,8 +571,8 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   }
   if (rc == POLYMUL_OK) apply_candidate(p, 0);
   if (rc == POLYMUL_OK && few) {
-    p->other.cand = few;
     const uint64_t sms = (uint64_t)p->num_sms;
+    p->other.cand = few;
     if (p->elem == 8) {
       p->other.upto = sms >> (p->logn - 12);  // 76, 38, 19 products at 2^13, 2^14, 2^15
     } else if (p->logn == 14) {
@@ -576,26 +581,23 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
       // The 128-register kernel beside the 64-register default.  2^13, one
       // product per SM at most: nothing else runs beside it, and 128 registers
       // hold more loads in flight (125 products, q < 2^20: 12.7 us against
-      // 13.3).  Overlapped batches: the next one's CTAs start as this one's
-      // leave, and with fewer resident CTAs, each taking several products, they
-      // fill the SMs evenly, where the default runs in whole waves of two CTAs
-      // per SM at 2^13, four at 2^12 (2^13, q < 2^30, default / this, batches
-      // of 156 20.4 / 15.9 us, 230 20.7 / 17.7, 304 20.8 / 21.7, 320 29.1 /
-      // 23.0, 410 32.0 / 29.4, 480 35.9 / 34.2, 520 35.5 / 36.8; 2^12, 500
-      // 17.1 / 15.3, 830 26.5 / 23.7, 1216 36.5 / 33.5, 1600 43.6 / 44.1).
-      if (p->logn == 13) {
-        p->other.upto = overlap ? 15 * sms / 8 : sms;
-        if (overlap) p->other.lo = 2 * sms, p->other.hi = 13 * sms / 4;
-      } else if (overlap) {
-        p->other.upto = 9 * sms;
-      } else if (p->mode == 2) {
-        // the unreduced mode multiplies less, and latency weighs more (q < 2^17,
-        // 2^12, default / this: 20 products 8.0 / 7.6 us, 360 15.2 / 14.6, 450
-        // 15.4 / 15.3, 500 18.8 / 19.6)
-        p->other.upto = 3 * sms;
-      }
+      // 13.3).  2^12 in the unreduced mode: it multiplies less, and latency
+      // weighs more (q < 2^17, default / this: 20 products 8.0 / 7.6 us, 360
+      // 15.2 / 14.6, 450 15.4 / 15.3, 500 18.8 / 19.6).
+      if (p->logn == 13) p->other.upto = sms;
+      if (p->logn == 12 && p->mode == 2) p->other.upto = 3 * sms;
+      // Batches that run ahead: the next one's CTAs start as this one's leave,
+      // and with fewer resident CTAs, each taking several products, they fill
+      // the SMs evenly, where the default runs in whole waves of two CTAs per SM
+      // at 2^13, four at 2^12 (2^13, q < 2^30, default / this, batches of 156
+      // 20.4 / 15.9 us, 230 20.7 / 17.7, 304 20.8 / 21.7, 320 29.1 / 23.0, 410
+      // 32.0 / 29.4, 480 35.9 / 34.2, 520 35.5 / 36.8; 2^12, 500 17.1 / 15.3,
+      // 830 26.5 / 23.7, 1216 36.5 / 33.5, 1600 43.6 / 44.1).
+      p->ahead = p->logn == 13 ? BatchRule{few, 15 * sms / 8, 2 * sms, 13 * sms / 4} : BatchRule{few, 9 * sms, 0, 0};
     } else {
       p->other.upto = sms * 2048 / p->n;
+      // larger batches that run ahead: one operand in registers at a time
+      if (one_operand) p->ahead = BatchRule{one_operand, 0, p->other.upto, UINT64_MAX};
     }
   }
   // Small batches leave most of the GPU idle whatever the kernel: one unit's
@@ -605,18 +607,20 @@ extern "C" int polymul_create(uint32_t n, const uint64_t* q_list, uint32_t k, co
   // two meet (n = 512, 1216 units: 8.9 / 8.4).  Smallest moduli: the radix-16
   // kernel (n = 1024, 64 units: 5.4 us against 6.9; n = 256, 152 units:
   // 5.0 / 6.5) up to 4800 per SM, 4600 at n = 1024 (n = 256, 2850 units 7.4 /
-  // 8.4, 3265 9.6 / 8.4; n = 1024, 682 units 8.3 / 8.8, 712 8.3 / 8.0), in
-  // overlapped batches up to 4500 (n = 256, 2731 units 5.6 / 5.2), and at n =
-  // 256 where the tiny unit's second CTA on some SMs does not pay yet (32 units
-  // per CTA; 5343 units 9.9 / 10.2, 6234 10.5 / 10.3).
+  // 8.4, 3265 9.6 / 8.4; n = 1024, 682 units 8.3 / 8.8, 712 8.3 / 8.0), and at
+  // n = 256 where the tiny unit's second CTA on some SMs does not pay yet (32
+  // units per CTA; 5343 units 9.9 / 10.2, 6234 10.5 / 10.3); batches that run
+  // ahead only up to 4500 (n = 256, 2731 units 5.6 / 5.2).
   if (rc == POLYMUL_OK && p->cands.size() > 1 && (p->aux_prime || p->cands[0].ki.tiny)) {
     const uint64_t sms = (uint64_t)p->num_sms;
-    const uint64_t per_sm = p->aux_prime ? 3500 : overlap ? 4500 : p->n == 1024 ? 4600 : 4800;
-    p->other.cand = 1;
-    p->other.upto = sms * per_sm / p->n;
-    if (!p->aux_prime && !overlap && p->n == 256) p->other.lo = 32 * sms, p->other.hi = 39 * sms;
+    p->other = BatchRule{1, sms * (p->aux_prime ? 3500 : p->n == 1024 ? 4600 : 4800) / p->n, 0, 0};
+    p->ahead = BatchRule{};
+    if (!p->aux_prime) {
+      if (p->n == 256) p->other.lo = 32 * sms, p->other.hi = 39 * sms;
+      p->ahead = BatchRule{0, 0, sms * 4500 / p->n, UINT64_MAX};
+    }
   }
-  p->other_on = p->other.upto > 0;
+  p->rules_on = p->other.upto > 0 || p->ahead.hi > 0 || p->ahead.upto > 0;
   if (rc == POLYMUL_OK) {
     // work counters for the three launch slots (device entry, two host-entry streams)
     if (cudaMalloc(&p->d_ctr, 2 * kCounterSlots * sizeof(unsigned long long)) != cudaSuccess ||
@@ -826,13 +830,22 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     const int r = validate_operands(p, a, b, units, st);
     if (r != POLYMUL_OK) return r;
   }
-  // the kernel: the plan's choice, or the candidate for batches of this size
-  // (a pending diagnostics injection counts launches of the batch kernel, so
-  // it keeps the plan's choice)
-  const PlanCandidate* other =
-      p->other_on && p->other.takes(units) && !injected_wait_pending() ? &p->cands[p->other.cand] : nullptr;
-  const KernelInfo& ki = other ? other->ki : p->ki;
-  const int grid_cap = other ? other->grid_cap : p->grid_cap;
+  // NTT batches: may this one start before its predecessor on the stream has
+  // finished (stream_order.h)?  The record's lock is held until the launch
+  const uintptr_t bytes = (uintptr_t)(units * p->n * p->elem);
+  LaunchFootprint fp;
+  fp.a_lo = (uintptr_t)a, fp.a_hi = (uintptr_t)a + bytes;
+  fp.b_lo = (uintptr_t)b, fp.b_hi = (uintptr_t)b + bytes;
+  fp.c_lo = (uintptr_t)c, fp.c_hi = (uintptr_t)c + bytes;
+  std::optional<StreamOrderGuard> order;
+  if (p->path == POLYMUL_PATH_NTT) order.emplace(p->device, st);
+  const bool runs_ahead = order && (p->flags & POLYMUL_FLAG_OVERLAP) && order->may_run_ahead(fp);
+  // the kernel: the plan's choice, or the candidate for such a batch (a pending
+  // diagnostics injection counts launches of the batch kernel, so it keeps the
+  // plan's choice)
+  const size_t which = injected_wait_pending() ? SIZE_MAX : p->candidate_for(units, runs_ahead);
+  const KernelInfo& ki = which == SIZE_MAX ? p->ki : p->cands[which].ki;
+  const int grid_cap = which == SIZE_MAX ? p->grid_cap : p->cands[which].grid_cap;
   const uint64_t need = (units + ki.units_per_cta - 1) / ki.units_per_cta;
   int grid = (int)std::min<uint64_t>(need, (uint64_t)grid_cap);
   int smem = ki.smem;
@@ -933,16 +946,9 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     PM_CUDA(cudaLaunchKernel(ki.fn, grid, ki.block, argv, ki.smem, st));
   } else {
     // the batch kernel: record its footprint for the next launch on this
-    // stream, and let it run ahead of the previous one where that is safe
-    // (stream_order.h); the cluster kernel takes no dependent launch
-    const uintptr_t bytes = (uintptr_t)(units * p->n * p->elem);
-    LaunchFootprint fp;
-    fp.a_lo = (uintptr_t)a, fp.a_hi = (uintptr_t)a + bytes;
-    fp.b_lo = (uintptr_t)b, fp.b_hi = (uintptr_t)b + bytes;
-    fp.c_lo = (uintptr_t)c, fp.c_hi = (uintptr_t)c + bytes;
-    StreamOrderGuard order(p->device, st);
-    const bool pdl = ki.cluster == 0 && (p->launch_flags & kLaunchPdl);
-    const uint32_t early = pdl && (p->flags & POLYMUL_FLAG_OVERLAP) && order.may_run_ahead(fp) ? 1u : 0u;
+    // stream, and let it run ahead of the previous one where that is safe;
+    // the cluster kernel takes no dependent launch
+    const uint32_t early = ki.cluster == 0 && (p->launch_flags & kLaunchPdl) && runs_ahead ? 1u : 0u;
     int r;
     uint32_t tx_pad = 0, polls = 0;
     if (ki.cluster == 0) take_injected_wait(&tx_pad, &polls);  // the cluster kernel has no copy waits
@@ -965,7 +971,7 @@ int launch_batch(polymul_plan* p, const void* a, const void* b, void* c, uint64_
     }
     // a failed launch enqueued nothing; a cluster launch lets its successor
     // start only at completion, but recording it is harmless
-    if (r == POLYMUL_OK) order.record(&fp);
+    if (r == POLYMUL_OK) order->record(&fp);
     return r;
   }
   return POLYMUL_OK;

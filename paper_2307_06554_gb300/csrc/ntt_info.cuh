@@ -19,11 +19,12 @@ constexpr int kNttWarps = 4;  // warps per CTA when a team fits in a warp
 //                                 primes, 3 M coefficients: 22.5 us at 2^10,
 //                                 both operands 23.6; 24.0 / 25.1 at 2^11),
 //                                 except
-//   ... Harvey's bounds:         both operands, without POLYMUL_FLAG_OVERLAP
-//                                 (q < 2^30, 3.2 M coefficients, one operand /
-//                                 both: 23.6 / 22.7 us at 2^10, 24.4 / 24.3 at
-//                                 2^11; overlapped 19.3 / 19.9 and 20.2 / 21.3:
-//                                 see lookup_ntt_u32_m1_seq);
+//   ... Harvey's bounds:         both operands, except in batches that run ahead
+//                                 of their predecessor (q < 2^30, 3.2 M
+//                                 coefficients, one operand / both: 23.6 / 22.7
+//                                 us at 2^10, 24.4 / 24.3 at 2^11; overlapped
+//                                 19.3 / 19.9 and 20.2 / 21.3: see
+//                                 polymul_create);
 //   32-bit words, n >= 2^12:     radix 16, padded, 64 registers, both operands:
 //                                 32 warps per SM hold the multiply pipe at
 //                                 74 % of its cycles.  16 M coefficients,

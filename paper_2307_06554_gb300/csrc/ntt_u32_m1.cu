@@ -16,8 +16,9 @@ bool lookup_ntt_u32_m1(int logn, KernelInfo* ki) {
   }
 }
 
-// One operand in registers at a time, for overlapped batches at 2^10, 2^11:
-// the faster shape there (see NttCfg), as the other modes' default is.
+// One operand in registers at a time, for batches at 2^10, 2^11 that run ahead
+// of their predecessor: the faster shape there (see NttCfg), as the other
+// modes' default is.
 bool lookup_ntt_u32_m1_seq(int logn, KernelInfo* ki) {
   if (logn == 10) *ki = ntt_info_x<uint32_t, 10, 1, false, 4, 96, 4, true>();
   if (logn == 11) *ki = ntt_info_x<uint32_t, 11, 1, false, 4, 96, 4, true>();

@@ -57,10 +57,17 @@ struct polymul_plan {
   std::vector<PlanCandidate> cands;  // [0] is the default
   size_t chosen = 0;
   // batches that run another candidate than the default one (see
-  // polymul_create); `other_on`: the rule holds, i.e. the choice is the
-  // default one and not an explicit one (polymul_plan_select)
-  BatchRule other;
-  bool other_on = false;
+  // polymul_create): by size, and, first, those that may start while their
+  // predecessor still runs (POLYMUL_FLAG_OVERLAP).  `rules_on`: the choice is
+  // the default one and not an explicit one (polymul_plan_select)
+  BatchRule other, ahead;
+  bool rules_on = false;
+  // the candidate of a batch, or SIZE_MAX: the plan's choice
+  size_t candidate_for(uint64_t units, bool runs_ahead) const {
+    if (!rules_on) return SIZE_MAX;
+    if (runs_ahead && ahead.takes(units)) return ahead.cand;
+    return other.takes(units) ? other.cand : SIZE_MAX;
+  }
   bool tuned = false;
   uint64_t tuned_batch = 0;  // batch bucket of the tuned choice
   void* d_tpc = nullptr;  // tensor-path constants
@@ -106,7 +113,7 @@ struct polymul_plan {
 
 inline void apply_candidate(polymul_plan* p, size_t i) {
   p->chosen = i;
-  p->other_on = false;
+  p->rules_on = false;
   p->path = p->cands[i].path;
   p->ki = p->cands[i].ki;
   p->grid_cap = p->cands[i].grid_cap;

@@ -81,7 +81,7 @@ std::string label_of(const PlanCandidate& c) {
 // sizes take, unless it was measured at such a size and won there.
 void settle(polymul_plan* p, size_t i, uint64_t bucket) {
   apply_candidate(p, i);
-  p->other_on = i == 0 && !p->other.takes(bucket * p->k);
+  p->rules_on = i == 0 && !p->other.takes(bucket * p->k);
   p->tuned = true;
   p->tuned_batch = bucket;
 }
@@ -145,7 +145,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
       cudaEventCreate(&e1) != cudaSuccess)
     rc = fail(POLYMUL_ECUDA, "tuning setup failed");
   const size_t saved_chosen = p->chosen;
-  const bool saved_other = p->other_on;
+  const bool saved_rules = p->rules_on;
   const uint32_t saved_flags = p->flags;
   p->flags &= ~POLYMUL_FLAG_VALIDATE;
   std::vector<float> best_ms(p->cands.size(), 1e30f);
@@ -196,7 +196,7 @@ extern "C" int polymul_tune(polymul_plan* p, uint64_t batch, void* stream) {
   cudaFree(buf);
   if (rc != POLYMUL_OK) {
     apply_candidate(p, saved_chosen);
-    p->other_on = saved_other;
+    p->rules_on = saved_rules;
     return rc;
   }
   settle(p, best, bucket);
