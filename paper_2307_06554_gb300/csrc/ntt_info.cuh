@@ -30,8 +30,11 @@ constexpr int kNttWarps = 4;  // warps per CTA when a team fits in a warp
 //                                 74 % of its cycles.  16 M coefficients,
 //                                 q < 2^31: 112.4 us at 2^12 (swizzled, 128
 //                                 registers: 123.0), 141.3 at 2^13 (164.6);
-//                                 8 M, q < 2^30, 2^12: 57.2 (62.0).  2^14 takes
-//                                 a 512-thread CTA of its own (ntt_u32_rb5.cu);
+//                                 8 M, q < 2^30, 2^12: 57.2 (62.0).  Few
+//                                 products and batches that run ahead of their
+//                                 predecessor take the 128-register kernel for
+//                                 some sizes (see polymul_create).  2^14 takes a
+//                                 512-thread CTA of its own (ntt_u32_rb5.cu);
 //   64-bit words, 2^6 .. 2^11:   radix 8, padded, 96 registers, one operand
 //                                 (radix 16 spills: 1.35-1.47x faster);
 //   64-bit words, 2^12:          radix 8, padded, 64 registers, both operands:
